@@ -4,8 +4,9 @@
 // One CTA owns up to ROWS query rows (tree node x query head of one kv head) and a
 // share of the key tiles (64 or 128 keys each).  Its warps (six, or ten with 128-row accumulators)
 // have three roles that only meet at mbarriers:
-//   warp 4 (loader)   brings K and V tiles (units K0 V0 K1 V1 ...) into a ring of five to eight
-//                     slots (UmmaCfg::SLOTS) in the 128-byte-swizzled layout the matrix descriptors
+//   warp 4 (loader)   brings K and V tiles (units K0 K1 V0 K2 V1 ..., the order in which the issuer
+//                     reads them: a slot is refilled as soon as the tile in it has been used) into
+//                     a ring of five to eight slots (UmmaCfg::SLOTS) in the 128-byte-swizzled layout the matrix descriptors
 //                     name: tiles that lie wholly in the cached prefix by TMA (two 64-column boxes of
 //                     a 5-D tensor map over the cache, completion counted on the slot's mbarrier),
 //                     the tile that holds the prefix end and the tree's own rows by 16-byte
@@ -47,7 +48,7 @@ namespace {
 constexpr int kD = 128;          // head_dim
 // warps 0-3 softmax, warp 4 loader, warp 5 MMA issuer; with 128-row accumulators warps 6-9 are a
 // second softmax group (UmmaCfg::THREADS)
-constexpr int kMaxSlots = 8;                      // ring of K / V tiles (K0 V0 K1 V1 K2 ...)
+constexpr int kMaxSlots = 8;                      // ring of K / V tiles (K0 K1 V0 K2 V1 ...)
 constexpr float kLazyMax = 8.f;                   // raise the running max only beyond this (log2 units)
 
 // KT = keys per tile: 64 (two CTAs per SM, 256 tensor-memory columns each) or 128 (one CTA per SM
@@ -161,13 +162,21 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap km
   }
   // every exit before the key loop hands the tensor memory back
   auto leave = [&]() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");     // (the next kernel only waits for this one)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (warp == 5) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(C::TMEM_COLS) : "memory");
   };
 
-  grid_dependency_sync();
+  // Normally nothing is read before the preceding kernel of the stream has completed.  With
+  // `early_prefix` the caller has promised that it writes neither the lengths, the parent array nor
+  // cache rows below kv_len: those are read, and the first ring of prefix tiles is requested, while it
+  // is still draining; every thread waits for it before it touches q, the tree's rows or the output.
+  // (This is what lets the launches of a call chain flow into each other: CTAs of the next launch
+  // start in the slots that this launch's last wave leaves empty.)
+  auto wait_predecessor = [&]() { asm volatile("griddepcontrol.wait;" ::: "memory"); };
+  if (!p.early_prefix) wait_predecessor();
   // ---- per-request metadata; every exit below is uniform over the cluster ----
   const int n = p.n_nodes[b], L = p.kv_len[b];
   const int my_parent = tid < p.t_max ? p.parent[(long long)b * p.t_max + tid] : -1;
@@ -219,6 +228,12 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap km
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // (only now, with this CTA's tensor memory allocated, may CTAs of the next kernel be scheduled: they
+  // could take the columns and then wait for this kernel to complete)
+  if (!p.early_prefix || warp != 4) {
+    wait_predecessor();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   const uint32_t tmem = s_tmem;
   const uint32_t tmem_o = tmem + C::O_COL;
   volatile int *fail = &s_fail;
@@ -268,21 +283,26 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap km
     };
     const int n_units = 2 * n_my;
     bool ok = true;
+    // unit u: K0, then K(t) and V(t-1) in turn, V of the last tile
+    auto is_v = [&](int u) { return u > 0 && (!(u & 1) || u == n_units - 1); };
+    auto tile_of = [&](int u) { return t_begin + (u == n_units - 1 ? n_my - 1 : (u & 1) ? (u + 1) >> 1 : u == 0 ? 0 : (u >> 1) - 1); };
+    auto in_prefix = [&](int u) { return tile_of(u) * KT + KT <= L; };
     auto issue_unit = [&](int u) {
       const int slot = u % kSlots;
-      const int t = t_begin + (u >> 1);
+      const int t = tile_of(u);
+      const bool value = is_v(u);
       const uint32_t dst = ring_s + slot * kTileBytes;
       if (t * KT + KT <= L) {                   // whole tile inside the cached prefix: two TMA boxes
         if (lane == 0) {
           mbar_arrive_expect_tx(bar_full(slot), kTileBytes);
-          const CUtensorMap *map = (u & 1) ? &vmap : &kmap;
+          const CUtensorMap *map = value ? &vmap : &kmap;
           tma_load_5d(dst, map, bar_full(slot), 0, t * KT, hk, b, p.layer);
           tma_load_5d(dst + kPanelBytes, map, bar_full(slot), 64, t * KT, hk, b, p.layer);
         } else {
           mbar_arrive(bar_full(slot));
         }
       } else {                                  // prefix end and / or tree rows: cp.async with zero fill
-        const __nv_bfloat16 *cbase = (u & 1) ? cv : ck, *tbase = (u & 1) ? tv : tk;
+        const __nv_bfloat16 *cbase = value ? cv : ck, *tbase = value ? tv : tk;
 #pragma unroll 4
         for (int i = 0; i < KT / 2; ++i) {
           const int r = rbase + 2 * i;
@@ -308,11 +328,20 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap km
         mbar_arrive(bar_full(slot));
       }
     };
-    // K of the first tile, then Q (what S(0) needs), then the rest of the first ring
+    // K of the first tile, then Q (what S(0) needs), then the rest of the first ring; with early_prefix
+    // the whole first ring, as far as it lies in the cached prefix, before the wait that Q needs
     const int n_first = min(n_units, kSlots);
-    if (n_first > 0) issue_unit(0);
+    if (p.early_prefix) {
+      for (int u = 0; u < n_first; ++u)
+        if (in_prefix(u)) issue_unit(u);
+      wait_predecessor();
+      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    } else if (n_first > 0) {
+      issue_unit(0);
+    }
     if (n_my > 0 && !C::TMEM_AB) issue_q();
-    for (int u = 1; u < n_first; ++u) issue_unit(u);
+    for (int u = p.early_prefix ? 0 : 1; u < n_first; ++u)
+      if (!p.early_prefix || !in_prefix(u)) issue_unit(u);
     for (int u = n_first; u < n_units && ok; ++u) {
       publish_q();                              // (all ring slots are in flight by now)
       ok = mbar_wait(bar_empty(u % kSlots), (u / kSlots - 1) & 1, fail);
@@ -332,7 +361,7 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap km
         tc_fence_after();
       };
       auto issue_s = [&](int it) {            // S(it) = Q K(it)^T into S buffer it & 1
-        const int u = 2 * it;
+        const int u = it == 0 ? 0 : 2 * it - 1;
         wait_full(u);
         if (!ok) return;
         const uint32_t kb = ring_s + (u % kSlots) * kTileBytes;
@@ -355,7 +384,7 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap km
       }
       if (n_my > 1) issue_s(1);
       for (int it = 0; it < n_my && ok; ++it) {
-        const int u = 2 * it + 1;
+        const int u = it == n_my - 1 ? 2 * n_my - 1 : 2 * it + 2;
         const int pb = it % PB;
         ok = mbar_wait(bar_p(pb), (it / PB) & 1, fail);   // P(it) is in shared memory, S(it) has been read
         wait_full(u);
