@@ -710,11 +710,14 @@ extern "C" twig_status tree_verify_attention_ex(const void *q, const void *tree_
                                              : launch_tree_attn_umma(p, cache->batch, rows, st);
   }
   if (kernel == TWIG_ATTN_KERNEL_AUTO && umma_ok) {
-    // automatic choice: the tcgen05 kernel with cluster splits once there are more than 32 query rows
-    // per kv head or enough (request, kv head) pairs to fill the GPU, the mma.sync kernel for small,
-    // latency-bound calls.  (The persistent kernel measured slower than the cluster kernel on every
-    // shape tried, so it only runs when it is named.)
-    const bool big = rows > 32 || (long long)cache->batch * cache->n_kv_heads >= 148;
+    // automatic choice.  The mma.sync kernel is for small, latency-bound calls: few (request, kv head)
+    // pairs and few rows; there the host can only go by the cache's capacity (the lengths are on the
+    // device): at 32 rows and 32 pairs the two kernels cross near 800 keys (250 keys 5.8 against 7.6 us,
+    // 4000 keys 19.1 against 15.6), so capacities below 2048 keep it.  With more than 32 rows they cross
+    // at 250 keys; with more than 74 pairs the tcgen05 kernels are never slower.  (The persistent
+    // kernel measured slower on every shape tried, so it only runs when it is named.)
+    const long long pairs = (long long)cache->batch * cache->n_kv_heads;
+    const bool big = pairs > 74 || rows > 64 || cache->max_len >= (rows > 32 ? 256 : 2048);
     if (big) {
       const twig_status us = launch_tree_attn_umma(p, cache->batch, rows, st);
       if (us != TWIG_ERR_UNSUPPORTED) return us;     // no tensor map for this layout: the mma.sync kernel

@@ -144,9 +144,13 @@ struct CacheMaps {
   alignas(64) CUtensorMap vmap;
 };
 bool cache_maps(const AttnParams &p, int box_rows, CacheMaps *out);
+// The same over the call's tree rows, dims (d, node, request x head); encoded on every call.
+bool tree_maps(const AttnParams &p, int box_rows, CacheMaps *out);
 
 // tcgen05 path (tree_attn_umma.cu): head_dim 128, rows = t_max * group.
 twig_status launch_tree_attn_umma(AttnParams &p, int batch, int rows, cudaStream_t st);
+// the same for rows <= 64, products transposed (tree_attn_narrow.cu)
+twig_status launch_tree_attn_narrow(AttnParams &p, int batch, int rows, cudaStream_t st);
 // persistent tcgen05 path (tree_attn_stream.cu): the same shapes, needs the caller's scratch
 twig_status launch_tree_attn_stream(AttnParams &p, int batch, int rows, cudaStream_t st);
 size_t tree_attn_stream_workspace_bytes(int batch, int n_q_heads, int max_nodes);

@@ -896,6 +896,18 @@ struct MapEntry {
   alignas(64) CUtensorMap vmap;
   bool valid = false;
 };
+constexpr int kMapEntries = 32;      // (a cache in use takes up to three entries)
+
+static EncodeTiledFn encode_tiled() {
+  static const EncodeTiledFn fn = []() -> EncodeTiledFn {
+    void *ptr = nullptr;
+    cudaDriverEntryPointQueryResult qres;
+    const bool found = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
+                       qres == cudaDriverEntryPointSuccess;
+    return found ? reinterpret_cast<EncodeTiledFn>(ptr) : nullptr;
+  }();
+  return fn;
+}
 
 static bool encode_cache_map(EncodeTiledFn fn, CUtensorMap *out, const void *base, const MapKey &key) {
   const cuuint64_t dims[5] = {(cuuint64_t)kD, (cuuint64_t)key.max_len, (cuuint64_t)key.heads, (cuuint64_t)key.batch,
@@ -916,20 +928,11 @@ static bool encode_cache_map(EncodeTiledFn fn, CUtensorMap *out, const void *bas
 // the caller gets a copy, not a pointer into it.)
 bool cache_maps(const AttnParams &p, int box_rows, CacheMaps *out) {
   static std::mutex mu;
-  static EncodeTiledFn fn = nullptr;
-  static bool fn_tried = false;
-  static MapEntry table[16];
+  static MapEntry table[kMapEntries];
   static int next = 0;
-  std::lock_guard<std::mutex> lock(mu);
-  if (!fn_tried) {
-    fn_tried = true;
-    void *ptr = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(ptr);
-  }
+  const EncodeTiledFn fn = encode_tiled();
   if (!fn) return false;
+  std::lock_guard<std::mutex> lock(mu);
   // strides must be multiples of 16 bytes, and every dimension but the last needs stride * extent in range
   if (p.c_sp <= 0 || p.c_sh <= 0 || p.c_sb < 0 || p.c_sl < 0) return false;
   MapKey key{p.cache_k0, p.cache_v0, p.n_layers > 1 ? p.c_sl : p.c_sp, p.batch > 1 ? p.c_sb : p.c_sp, p.c_sh, p.c_sp,
@@ -942,7 +945,7 @@ bool cache_maps(const AttnParams &p, int box_rows, CacheMaps *out) {
       return true;
     }
   MapEntry &e = table[next];
-  next = (next + 1) % 16;
+  next = (next + 1) % kMapEntries;
   e.valid = false;
   if (!encode_cache_map(fn, &e.kmap, p.cache_k0, key) || !encode_cache_map(fn, &e.vmap, p.cache_v0, key)) return false;
   e.key = key;
@@ -950,6 +953,20 @@ bool cache_maps(const AttnParams &p, int box_rows, CacheMaps *out) {
   out->kmap = e.kmap;
   out->vmap = e.vmap;
   return true;
+}
+
+bool tree_maps(const AttnParams &p, int box_rows, CacheMaps *out) {
+  const EncodeTiledFn fn = encode_tiled();
+  if (!fn) return false;
+  const cuuint64_t dims[3] = {(cuuint64_t)kD, (cuuint64_t)p.t_max, (cuuint64_t)p.batch * p.n_kv_heads};
+  const cuuint64_t strides[2] = {(cuuint64_t)kD * 2, (cuuint64_t)kD * 2 * p.t_max};
+  const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1}, estr[3] = {1, 1, 1};
+  auto encode = [&](CUtensorMap *map, const __nv_bfloat16 *base) {
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16 *>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  return encode(&out->kmap, p.tree_k) && encode(&out->vmap, p.tree_v);
 }
 
 namespace {
@@ -986,6 +1003,7 @@ twig_status launch_umma(const AttnParams &p, const CacheMaps *maps, int batch, i
 }  // namespace
 
 twig_status launch_tree_attn_umma(AttnParams &p, int batch, int rows, cudaStream_t st) {
+  if (rows <= 64) return launch_tree_attn_narrow(p, batch, rows, st);
   const int rows_per_cta = rows <= 32 ? 32 : rows <= 64 ? 64 : 128;
   p.row_blocks = (rows + rows_per_cta - 1) / rows_per_cta;
   if ((long long)p.n_kv_heads * p.row_blocks > 65535) return TWIG_ERR_UNSUPPORTED;
