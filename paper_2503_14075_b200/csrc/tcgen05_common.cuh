@@ -43,6 +43,62 @@ __device__ __forceinline__ void umma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64
       ::"r"(tmem_d), "r"(tmem_a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// ---- products of eight steps of K = 16, issued by a whole warp in uniform control flow ----
+// `leader` is the predicate of one elected lane.  The descriptors stay in uniform registers and advance by
+// constants: with one lane in divergent code the compiler rebuilt and moved them for every instruction, and
+// eight instructions took 770 to 1020 cycles to issue where they run 512.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r;
+}
+// one step's descriptor advance (in 16-byte units): K-major operand of two 64-column panels; MN-major operand
+#define TWIG_MMA_SS(acc) "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, " acc ";\n\t"
+#define TWIG_MMA_TS(acc) "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [t], b, %3, " acc ";\n\t"
+#define TWIG_STEP(x, y) "add.s64 a, a, " x ";\n\tadd.s64 b, b, " y ";\n\t"
+// D (+)= A B, both operands K-major in shared memory, two panels PA / PB bytes apart
+template <int PA, int PB>
+__device__ __forceinline__ void umma8_kk(uint32_t leader, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
+  asm volatile(
+      "{\n\t.reg .pred p, q, t;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 q, %4, 0;\n\tsetp.ne.b32 t, 1, 0;\n\tsetp.ne.b32 p, 0, 0;\n\t"
+      "mov.b64 a, %1;\n\tmov.b64 b, %2;\n\t"
+      TWIG_MMA_SS("p") TWIG_STEP("2", "2") TWIG_MMA_SS("t") TWIG_STEP("2", "2") TWIG_MMA_SS("t") TWIG_STEP("2", "2") TWIG_MMA_SS("t")
+      TWIG_STEP("%5", "%6")
+      TWIG_MMA_SS("t") TWIG_STEP("2", "2") TWIG_MMA_SS("t") TWIG_STEP("2", "2") TWIG_MMA_SS("t") TWIG_STEP("2", "2") TWIG_MMA_SS("t") "}"
+      ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(leader), "n"((PA >> 4) - 6), "n"((PB >> 4) - 6) : "memory");
+}
+// D (+)= A B, operands that advance by SA / SB bytes a step; `accumulate`: whether the first step adds to D
+template <int SA, int SB>
+__device__ __forceinline__ void umma8_ss(uint32_t leader, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q, t;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 q, %4, 0;\n\tsetp.ne.b32 t, 1, 0;\n\tsetp.ne.b32 p, %7, 0;\n\t"
+      "mov.b64 a, %1;\n\tmov.b64 b, %2;\n\t"
+      TWIG_MMA_SS("p") TWIG_STEP("%5", "%6") TWIG_MMA_SS("t") TWIG_STEP("%5", "%6") TWIG_MMA_SS("t") TWIG_STEP("%5", "%6") TWIG_MMA_SS("t")
+      TWIG_STEP("%5", "%6")
+      TWIG_MMA_SS("t") TWIG_STEP("%5", "%6") TWIG_MMA_SS("t") TWIG_STEP("%5", "%6") TWIG_MMA_SS("t") TWIG_STEP("%5", "%6") TWIG_MMA_SS("t") "}"
+      ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(leader), "n"(SA >> 4), "n"(SB >> 4), "r"(accumulate) : "memory");
+}
+// D (+)= A B with A in tensor memory (eight columns a step), B advancing by SB bytes a step
+template <int SB>
+__device__ __forceinline__ void umma8_ts(uint32_t leader, uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+#define TWIG_STEP_TS "add.u32 t, t, 8;\n\tadd.s64 b, b, %5;\n\t"
+  asm volatile(
+      "{\n\t.reg .pred p, q, y;\n\t.reg .b64 b;\n\t.reg .b32 t;\n\tsetp.ne.b32 q, %4, 0;\n\tsetp.ne.b32 y, 1, 0;\n\tsetp.ne.b32 p, %6, 0;\n\t"
+      "mov.b32 t, %1;\n\tmov.b64 b, %2;\n\t"
+      TWIG_MMA_TS("p") TWIG_STEP_TS TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y")
+      TWIG_STEP_TS
+      TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y") "}"
+      ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(leader), "n"(SB >> 4), "r"(accumulate) : "memory");
+#undef TWIG_STEP_TS
+}
+#undef TWIG_MMA_SS
+#undef TWIG_MMA_TS
+#undef TWIG_STEP
+__device__ __forceinline__ void umma_commit_if(uint32_t leader, uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(leader) : "memory");
+}
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
@@ -132,6 +188,48 @@ __device__ __forceinline__ float poly_exp2(float x) {
   r = fmaf(r, f, 0.6931472f);
   r = fmaf(r, f, 1.f);
   return __int_as_float(__float_as_int(r) + (__float_as_int(t) << 23));   // * 2^n (the magic's bits shift out)
+}
+
+// ---- pairs of fp32 in one register pair: one instruction for two elements ----
+struct F2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float lo, float hi) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack(F2 a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+// poly_exp2 of both elements
+__device__ __forceinline__ F2 poly_exp2(F2 x) {
+  const float2 c = unpack(x);
+  x = f2(fmaxf(c.x, -126.f), fmaxf(c.y, -126.f));
+  const F2 magic = f2(12582912.f, 12582912.f), t = add2(x, magic);
+  const F2 f = add2(x, fma2(t, f2(-1.f, -1.f), magic));
+  F2 r = fma2(f, f2(0.0555041f, 0.0555041f), f2(0.2402265f, 0.2402265f));
+  r = fma2(r, f, f2(0.6931472f, 0.6931472f));
+  r = fma2(r, f, f2(1.f, 1.f));
+  const float2 rr = unpack(r), tt = unpack(t);
+  return f2(__int_as_float(__float_as_int(rr.x) + (__float_as_int(tt.x) << 23)), __int_as_float(__float_as_int(rr.y) + (__float_as_int(tt.y) << 23)));
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
 }
 
 }  // namespace twig

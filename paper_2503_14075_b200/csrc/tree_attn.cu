@@ -707,7 +707,7 @@ extern "C" twig_status tree_verify_attention_ex(const void *q, const void *tree_
   if (kernel == TWIG_ATTN_KERNEL_TCGEN05 || kernel == TWIG_ATTN_KERNEL_STREAM) {
     if (!umma_ok) return TWIG_ERR_UNSUPPORTED;
     return kernel == TWIG_ATTN_KERNEL_STREAM ? launch_tree_attn_stream(p, cache->batch, rows, st)
-                                             : launch_tree_attn_umma(p, cache->batch, rows, st);
+                                             : launch_tree_attn_tcgen05(p, cache->batch, rows, st);
   }
   if (kernel == TWIG_ATTN_KERNEL_AUTO && umma_ok) {
     // automatic choice.  The mma.sync kernel is for small, latency-bound calls: few (request, kv head)
@@ -719,7 +719,7 @@ extern "C" twig_status tree_verify_attention_ex(const void *q, const void *tree_
     const long long pairs = (long long)cache->batch * cache->n_kv_heads;
     const bool big = pairs > 74 || rows > 64 || cache->max_len >= (rows > 32 ? 256 : 2048);
     if (big) {
-      const twig_status us = launch_tree_attn_umma(p, cache->batch, rows, st);
+      const twig_status us = launch_tree_attn_tcgen05(p, cache->batch, rows, st);
       if (us != TWIG_ERR_UNSUPPORTED) return us;     // no tensor map for this layout: the mma.sync kernel
     }
   }

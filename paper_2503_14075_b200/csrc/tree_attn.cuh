@@ -147,8 +147,8 @@ bool cache_maps(const AttnParams &p, int box_rows, CacheMaps *out);
 // The same over the call's tree rows, dims (d, node, request x head); encoded on every call.
 bool tree_maps(const AttnParams &p, int box_rows, CacheMaps *out);
 
-// tcgen05 path (tree_attn_umma.cu): head_dim 128, rows = t_max * group.
-twig_status launch_tree_attn_umma(AttnParams &p, int batch, int rows, cudaStream_t st);
+// tcgen05 path (tree_attn_wide.cu): head_dim 128, rows = t_max * group.
+twig_status launch_tree_attn_tcgen05(AttnParams &p, int batch, int rows, cudaStream_t st);
 // the same for rows <= 64, products transposed (tree_attn_narrow.cu)
 twig_status launch_tree_attn_narrow(AttnParams &p, int batch, int rows, cudaStream_t st);
 // persistent tcgen05 path (tree_attn_stream.cu): the same shapes, needs the caller's scratch

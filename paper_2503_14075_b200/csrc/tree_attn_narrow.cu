@@ -26,7 +26,7 @@
 
 #include <type_traits>
 
-#include "tcgen05_common.cuh"
+#include "attn_tiles.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -35,9 +35,7 @@ namespace twig {
 namespace {
 
 constexpr int kD = 128;                            // head_dim
-constexpr int kKeys = 128;                         // keys per tile
-constexpr int kTileBytes = kKeys * kD * 2;         // one K (or V) tile: two 64-column panels
-constexpr int kPanelBytes = kKeys * 128;
+constexpr int kKeys = kTileKeys;                  // keys per tile
 constexpr int kThreads = 320;
 constexpr int kSoftWarps = 8;
 constexpr float kLazyMax = 8.f;                    // raise a row's reference only beyond this (log2 units)
@@ -133,19 +131,11 @@ __device__ __forceinline__ bool bar_any(int id, int threads, bool mine) {
       : "memory");
   return any != 0;
 }
-// one box of a 3-D tensor map (x, node, request x head)
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int node, int slice) {
-  asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-               ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(node), "r"(slice) : "memory");
-}
 // maximum over the warp
 __device__ __forceinline__ float warp_max(float x) {
   float y;
   asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
   return y;
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 // bytes of this CTA's shared memory -> a cluster CTA's, counted on that CTA's barrier
 __device__ __forceinline__ void bulk_to_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
@@ -153,14 +143,9 @@ __device__ __forceinline__ void bulk_to_cluster(uint32_t dst, uint32_t src, uint
                "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-// K and V: the cache in boxes of 128, 32 and 8 rows, the tree's rows in boxes of 8
-struct NarrowMaps {
-  CacheMaps whole, box32, box8, tree8;
-};
-
 template <int R, int SLOTS, int MIN_CTAS>
 __global__ void __launch_bounds__(kThreads, MIN_CTAS)
-tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ NarrowMaps maps) {
+tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps maps) {
   using C = NarrowCfg<R, SLOTS, MIN_CTAS>;
   using RowBits = typename std::conditional<R == 64, unsigned long long, unsigned int>::type;
   constexpr int RH = C::RH;
@@ -174,7 +159,8 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ NarrowMaps m
   __shared__ int s_fail;
 
   cg::cluster_group cluster = cg::this_cluster();
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // (uniform for the compiler too: see umma8_kk)
   const int split = blockIdx.x, n_splits = gridDim.x;
   const int hk = blockIdx.y / p.row_blocks, rb = blockIdx.y % p.row_blocks;
   const int b = blockIdx.z;
@@ -264,17 +250,10 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ NarrowMaps m
   auto unit_is_v = [&](int u) { return u > 0 && (!(u & 1) || u == n_units - 1); };
   auto unit_tile = [&](int u) { return t_begin + (u == n_units - 1 ? n_my - 1 : (u & 1) ? (u + 1) >> 1 : u == 0 ? 0 : (u >> 1) - 1); };
   auto unit_in_prefix = [&](int u) { return unit_tile(u) * kKeys + kKeys <= L; };
-  auto load_whole = [&](int u) {                   // a tile that lies in the cached prefix: two boxes
-    const int slot = u % SLOTS, t = unit_tile(u);
-    const uint32_t dst = ring_s + slot * kTileBytes;
-    if (lane == 0) {
-      const CUtensorMap *map = unit_is_v(u) ? &maps.whole.vmap : &maps.whole.kmap;
-      mbar_arrive_expect_tx(bar_full(slot), kTileBytes);
-      tma_load_5d(dst, map, bar_full(slot), 0, t * kKeys, hk, b, p.layer);
-      tma_load_5d(dst + kPanelBytes, map, bar_full(slot), 64, t * kKeys, hk, b, p.layer);
-    } else {
-      mbar_arrive(bar_full(slot));
-    }
+  const TileSource source{L, L8, NK, hk, b, p.layer, b * p.n_kv_heads + hk};
+  auto load_whole = [&](int u) {
+    const int slot = u % SLOTS;
+    load_whole_tile(maps, source, unit_is_v(u), ring_s + slot * kTileBytes, bar_full(slot), unit_tile(u) * kKeys, lane);
   };
   const int n_first = min(n_units, C::PRE_UNITS);
   if (warp == 8)
@@ -298,50 +277,6 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ NarrowMaps m
   if (warp == 8) {
     // ================= loader =================
     uint32_t raw_phase = 0;
-    auto load_edge = [&](int u) {                  // the tile that holds the prefix end and / or tree rows
-      const int slot = u % SLOTS, k0 = unit_tile(u) * kKeys;
-      const bool value = unit_is_v(u);
-      const uint32_t dst = ring_s + slot * kTileBytes;
-      const int pre = min(max(L8 - k0, 0), kKeys), tree0 = max(k0 - L8, 0);
-      const int n_tree = min(kKeys - pre, NK - L8 - tree0);            // tree rows of this tile
-      // rows of V between the prefix end and the tree, and after the tree up to the next multiple of 16 (the
-      // product's step in keys), must be zero: they are cleared once the boxes have landed
-      const bool clear = value;
-      const uint32_t bar = clear ? bar_raw : bar_full(slot);
-      const int e1 = pre >> 5, e2 = e1 + ((pre & 31) >> 3), e3 = e2 + ((n_tree + 7) >> 3);
-      if (lane == 0) {
-        const uint32_t bytes = (uint32_t)(pre + ((n_tree + 7) & ~7)) * kD * 2;
-        if (clear) mbar_arrive_expect_tx(bar, bytes);
-        else mbar_expect_tx(bar, bytes);
-      }
-      __syncwarp();
-      // boxes: prefix by 32 rows, by 8 rows, tree by 8 rows; both panels of each
-      for (int i = lane; i < 2 * e3; i += 32) {
-        const int x = (i & 1) * 64, j = i >> 1;
-        const uint32_t to = dst + (i & 1) * kPanelBytes;
-        if (j < e2) {
-          const int r = j < e1 ? 32 * j : (pre & ~31) + 8 * (j - e1);
-          const CacheMaps &m = j < e1 ? maps.box32 : maps.box8;
-          tma_load_5d(to + r * 128, value ? &m.vmap : &m.kmap, bar, x, k0 + r, hk, b, p.layer);
-        } else {
-          const int r = 8 * (j - e2);
-          tma_load_3d(to + (pre + r) * 128, value ? &maps.tree8.vmap : &maps.tree8.kmap, bar, x, tree0 + r, b * p.n_kv_heads + hk);
-        }
-      }
-      bool landed = true;
-      if (clear) {
-        landed = mbar_wait(bar_raw, raw_phase, fail);
-        raw_phase ^= 1;
-        const int g0 = min(max(L - k0, 0), kKeys), g1 = pre, t0 = pre + n_tree, t1 = min(kKeys, (t0 + 15) & ~15);
-        for (int i = lane; i < (g1 - g0 + t1 - t0) * 16; i += 32) {
-          const int q = i >> 4, r = q < g1 - g0 ? g0 + q : t0 + q - (g1 - g0);
-          asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(dst + ((i >> 3) & 1) * kPanelBytes + r * 128 + (i & 7) * 16), "r"(0u) : "memory");
-        }
-        fence_async_smem();
-      }
-      mbar_arrive(bar_full(slot));
-      return landed;
-    };
     bool ok = true;
     for (int u = 0; u < n_units && ok; ++u) {
       if (u < n_first && unit_in_prefix(u)) continue;      // requested above
@@ -353,37 +288,33 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ NarrowMaps m
       if (unit_in_prefix(u)) {
         load_whole(u);
       } else {
-        ok = load_edge(u);
+        ok = load_edge_tile(maps, source, unit_is_v(u), ring_s + u % SLOTS * kTileBytes, bar_full(u % SLOTS), bar_raw, raw_phase,
+                            unit_tile(u) * kKeys, lane, fail);
         ok = __all_sync(0xffffffffu, ok);
       }
     }
     if (!ok) s_fail = 1;
   } else if (warp == 9) {
-    // ================= MMA issuer (one thread) =================
-    if (lane == 0) {
+    // ================= MMA issuer (one elected lane; the warp stays together) =================
+    {
+      const uint32_t leader = elect_one();
       // S^T: A = K (K-major), B = Q (K-major); O^T: A = V (MN-major), B = P^T (MN-major)
       constexpr uint32_t kIdescS = instr_desc(128, R, false), kIdescO = instr_desc(128, R, true) | (1u << 15);
       bool ok = true;
       auto wait_full = [&](int u) {
         if (ok) ok = mbar_wait(bar_full(u % SLOTS), (u / SLOTS) & 1, fail);
-        fence_async_smem();
-        tc_fence_after();
       };
       auto issue_s = [&](int it) {
         const int u = it == 0 ? 0 : 2 * it - 1;
         wait_full(u);
         if (!ok) return;
-        const uint32_t kb = ring_s + (u % SLOTS) * kTileBytes;
-#pragma unroll
-        for (int ks = 0; ks < kD / 16; ++ks)
-          umma(tmem + (it & 1) * R, smem_desc(kb + (ks >> 2) * kPanelBytes + (ks & 3) * 32, 16),
-               smem_desc(q_s + (ks >> 2) * R * 128 + (ks & 3) * 32, 16), kIdescS, ks > 0);
-        umma_commit(bar_s(it & 1));
-        umma_commit(bar_empty(u % SLOTS));
+        umma8_kk<kPanelBytes, R * 128>(leader, tmem + (it & 1) * R, smem_desc(ring_s + (u % SLOTS) * kTileBytes, 16),
+                                       smem_desc(q_s, 16), kIdescS);
+        umma_commit_if(leader, bar_s(it & 1));
+        umma_commit_if(leader, bar_empty(u % SLOTS));
       };
       if (n_my > 0) {
         ok = mbar_wait(bar_q, 0, fail);
-        fence_async_smem();
         issue_s(0);
       }
       if (n_my > 1) issue_s(1);
@@ -392,19 +323,19 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ NarrowMaps m
         ok = mbar_wait(bar_p(it & 1), (it >> 1) & 1, fail);       // P(it) is in shared memory, S(it) has been read
         wait_full(u);
         if (!ok) break;
-        const uint32_t vb = ring_s + (u % SLOTS) * kTileBytes;
-        const uint32_t pb = p_s + it % C::P_BUFS * C::P_ONE;
+        tc_fence_after();
+        const uint64_t vd = smem_desc(ring_s + (u % SLOTS) * kTileBytes, kPanelBytes);
+        const uint64_t pd = smem_desc_of(p_s + it % C::P_BUFS * C::P_ONE, 16, 8 * C::P_ROW, C::P_LAYOUT);
         const int steps = (min(kKeys, NK - (t_begin + it) * kKeys) + 15) >> 4;     // 16 keys each
-#pragma unroll
-        for (int j = 0; j < kKeys / 16; ++j)
-          if (j < steps)
-            umma(tmem + C::O_COL, smem_desc(vb + j * 2048, kPanelBytes),
-                 smem_desc_of(pb + j * 16 * C::P_ROW, 16, 8 * C::P_ROW, C::P_LAYOUT), kIdescO, (it > 0) || (j > 0));
-        umma_commit(bar_o(it & 1));
-        umma_commit(bar_empty(u % SLOTS));
+        if (steps == kKeys / 16) umma8_ss<2048, 16 * C::P_ROW>(leader, tmem + C::O_COL, vd, pd, kIdescO, it > 0);
+        else
+          for (int j = 0; j < steps; ++j)
+            if (leader) umma(tmem + C::O_COL, vd + j * 128, pd + j * C::P_ROW, kIdescO, (it > 0) || (j > 0));
+        umma_commit_if(leader, bar_o(it & 1));
+        umma_commit_if(leader, bar_empty(u % SLOTS));
         if (it + 2 < n_my) issue_s(it + 2);
       }
-      if (!ok) s_fail = 1;
+      if (!ok && lane == 0) s_fail = 1;
     }
   } else {
     // ================= softmax: one key of a tile per thread, RH rows =================
@@ -665,7 +596,7 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ NarrowMaps m
 }
 
 template <int R, int SLOTS, int MIN_CTAS>
-twig_status launch_narrow(const AttnParams &p, const NarrowMaps &maps, int batch, int n_splits, cudaStream_t st) {
+twig_status launch_narrow(const AttnParams &p, const TileMaps &maps, int batch, int n_splits, cudaStream_t st) {
   using C = NarrowCfg<R, SLOTS, MIN_CTAS>;
   static bool attr_set = false;
   if (!attr_set) {
@@ -696,9 +627,8 @@ twig_status launch_narrow(const AttnParams &p, const NarrowMaps &maps, int batch
 twig_status launch_tree_attn_narrow(AttnParams &p, int batch, int rows, cudaStream_t st) {
   p.row_blocks = 1;
   if (p.n_kv_heads > 65535) return TWIG_ERR_UNSUPPORTED;
-  NarrowMaps maps;
-  if (!cache_maps(p, kKeys, &maps.whole) || !cache_maps(p, 32, &maps.box32) || !cache_maps(p, 8, &maps.box8) ||
-      !tree_maps(p, 8, &maps.tree8))
+  TileMaps maps;
+  if (!tile_maps(p, &maps))
     return TWIG_ERR_UNSUPPORTED;
   // Measured on chains of layers (us per launch, 32 kv heads; T nodes at L keys):
   //   at most 148 items: one CTA per SM with a deep ring, keys split over clusters below 75 items (T = 64, B = 4,
