@@ -78,16 +78,14 @@ __device__ __forceinline__ void umma8_ss(uint32_t leader, uint32_t d, uint64_t a
       TWIG_MMA_SS("t") TWIG_STEP("%5", "%6") TWIG_MMA_SS("t") TWIG_STEP("%5", "%6") TWIG_MMA_SS("t") TWIG_STEP("%5", "%6") TWIG_MMA_SS("t") "}"
       ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(leader), "n"(SA >> 4), "n"(SB >> 4), "r"(accumulate) : "memory");
 }
-// D (+)= A B with A in tensor memory (eight columns a step), B advancing by SB bytes a step
+// four steps of D (+)= A B with A in tensor memory (eight columns a step), B advancing by SB bytes a step
 template <int SB>
-__device__ __forceinline__ void umma8_ts(uint32_t leader, uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma4_ts(uint32_t leader, uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
 #define TWIG_STEP_TS "add.u32 t, t, 8;\n\tadd.s64 b, b, %5;\n\t"
   asm volatile(
       "{\n\t.reg .pred p, q, y;\n\t.reg .b64 b;\n\t.reg .b32 t;\n\tsetp.ne.b32 q, %4, 0;\n\tsetp.ne.b32 y, 1, 0;\n\tsetp.ne.b32 p, %6, 0;\n\t"
       "mov.b32 t, %1;\n\tmov.b64 b, %2;\n\t"
-      TWIG_MMA_TS("p") TWIG_STEP_TS TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y")
-      TWIG_STEP_TS
-      TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y") "}"
+      TWIG_MMA_TS("p") TWIG_STEP_TS TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y") TWIG_STEP_TS TWIG_MMA_TS("y") "}"
       ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(leader), "n"(SB >> 4), "r"(accumulate) : "memory");
 #undef TWIG_STEP_TS
 }

@@ -46,8 +46,8 @@ tree_attn_wide_kernel(const AttnParams p, const __grid_constant__ TileMaps maps)
   __shared__ unsigned long long s_mask[TWIG_MAX_NODES];       // ancestors-or-self of every node
   __shared__ int s_par[TWIG_MAX_NODES];
   __shared__ float2 s_pair[128];                              // (m, l) of stream 1's rows (same rows in both streams)
-  // full[kSlots], empty[kSlots], s[2], p[2], q[2], o[2], recv, raw
-  __shared__ __align__(8) unsigned long long s_bar[2 * kSlots + 10];
+  // full[kSlots], empty[kSlots], s[2], p[2 streams][2 halves], q[2], o[2], recv, raw
+  __shared__ __align__(8) unsigned long long s_bar[2 * kSlots + 12];
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
 
@@ -64,10 +64,11 @@ tree_attn_wide_kernel(const AttnParams p, const __grid_constant__ TileMaps maps)
   auto bar_full = [&](int slot) { return bars + 8 * slot; };
   auto bar_empty = [&](int slot) { return bars + 8 * (kSlots + slot); };
   auto bar_s = [&](int i) { return bars + 8 * (2 * kSlots + i); };
-  auto bar_p = [&](int i) { return bars + 8 * (2 * kSlots + 2 + i); };
-  auto bar_q = [&](int i) { return bars + 8 * (2 * kSlots + 4 + i); };
-  auto bar_o = [&](int i) { return bars + 8 * (2 * kSlots + 6 + i); };
-  const uint32_t bar_recv = bars + 8 * (2 * kSlots + 8), bar_raw = bars + 8 * (2 * kSlots + 9);
+  auto bar_p = [&](int i, int h) { return bars + 8 * (2 * kSlots + 2 + 2 * i + h); };
+  auto bar_q = [&](int i) { return bars + 8 * (2 * kSlots + 6 + i); };
+  auto bar_o = [&](int i) { return bars + 8 * (2 * kSlots + 8 + i); };
+  const uint32_t bar_recv = bars + 8 * (2 * kSlots + 10), bar_raw = bars + 8 * (2 * kSlots + 11);
+
   // ---- what needs nothing from global memory ----
   if (tid == 0) {
     s_fail = 0;
@@ -77,7 +78,8 @@ tree_attn_wide_kernel(const AttnParams p, const __grid_constant__ TileMaps maps)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar_s(i), 1);
-      mbar_init(bar_p(i), 4);                      // the stream's softmax warps
+      mbar_init(bar_p(i, 0), 4);                   // the stream's softmax warps
+      mbar_init(bar_p(i, 1), 4);
       mbar_init(bar_q(i), 4);
       mbar_init(bar_o(i), 1);
     }
@@ -224,17 +226,26 @@ tree_attn_wide_kernel(const AttnParams p, const __grid_constant__ TileMaps maps)
       if (ok && n_steps > 1) issue_s(1);
       for (int k = 0; k < n_steps && ok; ++k) {
         const int i = k & 1, t = tile_of(k), u = v_unit(t);
-        ok = mbar_wait(bar_p(i), (k >> 1) & 1, fail);         // P is in tensor memory
+        // P arrives in two halves of 64 keys: the product of the first runs while the softmax warps are still at
+        // the second (one piece: 3530 cycles per 128 keys of both streams)
+        ok = mbar_wait(bar_p(i, 0), (k >> 1) & 1, fail);
         if (!two || i == 0) wait_full(u);
         tc_fence_after();
         if (!ok) break;
         const uint64_t vd = smem_desc(ring_s + (u % kSlots) * kTileBytes, kPanelBytes);
         const int steps = (min(kKeys, NK - (t_begin + t) * kKeys) + 15) >> 4;     // 16 keys each
         const uint32_t o = tmem + 256 + i * 128, pt = tmem + i * 128;
-        if (steps == kKeys / 16) umma8_ts<2048>(leader, o, pt, vd, kIdescO, k > 1);
-        else
-          for (int j = 0; j < steps; ++j)
-            if (leader) umma_ts(o, pt + j * 8, vd + j * 128, kIdescO, k > 1 || j > 0);
+        auto product = [&](int h) {
+          if (steps >= 4 * h + 4) umma4_ts<2048>(leader, o, pt + h * 32, vd + h * 512, kIdescO, k > 1 || h > 0);
+          else
+            for (int j = 4 * h; j < steps; ++j)
+              if (leader) umma_ts(o, pt + j * 8, vd + j * 128, kIdescO, k > 1 || j > 0);
+        };
+        product(0);
+        ok = mbar_wait(bar_p(i, 1), (k >> 1) & 1, fail);
+        tc_fence_after();
+        if (!ok) break;
+        product(1);
         if (k + 2 >= n_steps) umma_commit_if(leader, bar_o(i));          // the stream's last product
         if (!two || i == 1) umma_commit_if(leader, bar_empty(u % kSlots));
         if (k + 2 < n_steps) issue_s(k + 2);
@@ -350,14 +361,22 @@ tree_attn_wide_kernel(const AttnParams p, const __grid_constant__ TileMaps maps)
             pw[c] = pack_bf16(pp.x, pp.y);
           }
           tmem_st32(ts + 32 * h, pw);
+          tmem_st_wait();
+          if (h == 0) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_p(stream, 0));
+          }
         }
-        tmem_st_wait();
         const float2 total = unpack(add2(sum[0], sum[1]));
         l_run += total.x + total.y;
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar_p(stream));
+      if (lane == 0) {
+        if (warp_idle) mbar_arrive(bar_p(stream, 0));
+        mbar_arrive(bar_p(stream, 1));
+      }
     }
     if (n_mine > 0) {
       ok = ok && mbar_wait(bar_o(stream), 0, fail);
