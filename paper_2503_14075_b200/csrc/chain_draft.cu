@@ -8,116 +8,57 @@
 // and acceptance take: a chain is a tree) and decides whether the request goes on drafting.
 // Requests that have stopped ignore further calls, so a batch can be driven through delta
 // calls without reading anything back.
-#include "twig_common.cuh"
+#include "vocab_row.cuh"
 
 namespace twig {
 
-constexpr int kChainThreads = 512;
-
-// running (maximum, its first index, sum of exp(x - maximum))
-struct MaxSum {
-  float m, s;
-  int i;
-};
-__device__ __forceinline__ void ms_take(MaxSum &a, float x, int i) {
-  if (x > a.m) {
-    a.s = a.s * __expf(a.m - x) + 1.f;      // (exp(-inf) = 0 for the first element)
-    a.m = x;
-    a.i = i;
-  } else if (x > -INFINITY) {                // (a logit of -inf adds nothing, also before any finite one)
-    a.s += __expf(x - a.m);
-  }
-}
-__device__ __forceinline__ void ms_merge(MaxSum &a, const MaxSum &b) {
-  if (b.m > a.m || (b.m == a.m && b.i < a.i)) {
-    a.s = b.s + a.s * __expf(a.m - b.m);
-    a.m = b.m;
-    a.i = b.i;
-  } else if (b.m > -INFINITY) {
-    a.s += b.s * __expf(b.m - a.m);
-  }
-}
-
+// Grid (slices, batch), clusters of the slices of a row.  One CTA per row took 13 us from a cold start at
+// 32000 fp32 logits (four round trips of loads, then one exponential after the other).
 template <bool FP32>
-__global__ void __launch_bounds__(kChainThreads)
+__global__ void __launch_bounds__(kRowThreads)
 chain_draft_step_kernel(const void *__restrict__ logits, long long row_stride, int vocab, int max_draft,
-                        float threshold, int *__restrict__ parent, int *__restrict__ draft_tok,
-                        float *__restrict__ tok_prob, int *__restrict__ n_nodes, int *__restrict__ active,
+                        float threshold, int *parent, int *draft_tok, float *tok_prob, int *n_nodes, int *active,
                         int t_max, int *dev_status) {
-  constexpr int EPC = FP32 ? 4 : 8;                 // elements per 16-byte chunk
-  __shared__ MaxSum s_part[kChainThreads / 32];
+  constexpr int EPC = RowFormat<FP32>::EPC;
+  __shared__ __align__(16) float4 s_peer[kMaxSlices];
+  __shared__ __align__(8) unsigned long long s_bar;
   grid_dependency_sync();
-  const int b = blockIdx.x, tid = threadIdx.x;
-  if (active[b] == 0) return;
+  const int b = blockIdx.y, tid = threadIdx.x;
+  SliceMerge sm{s_peer, smem_u32(&s_bar), (int)blockIdx.x, (int)gridDim.x};
+  const bool go = active[b] != 0;
   const int n = n_nodes[b];
-  if (n < 1 || n >= t_max) {                        // no root yet, or no room for another node
-    if (tid == 0) {
-      flag_status(dev_status, b, TWIG_DEV_BAD_TREE);
-      active[b] = 0;
-    }
+  if (!go) return;
+  const bool room = n >= 1 && n < t_max;            // a root, and room for another node
+  RowBest best{-INFINITY, 0.f, 0};
+  bool landed = true;
+  // (both words were read before the first CTA below can write them: it waits for its peers' results)
+  if (room) {
+    sm.start();
+    const unsigned char *row = static_cast<const unsigned char *>(logits) + (long long)b * row_stride * (FP32 ? 4 : 2);
+    const int chunks = vocab / EPC, per = (chunks + sm.slices - 1) / sm.slices;
+    best = scan_slice<FP32, true>(row, sm.rank * per, min(chunks, (sm.rank + 1) * per),
+                                  sm.rank == 0 && chunks * EPC < vocab, vocab);
+    landed = sm.merge<true>(best);
+  }
+  if (sm.rank > 0 || tid != 0) return;
+  if (!room || !landed) {
+    flag_status(dev_status, b, room ? TWIG_DEV_INTERNAL : TWIG_DEV_BAD_TREE);
+    active[b] = 0;
     return;
   }
-  const unsigned char *row = static_cast<const unsigned char *>(logits) + (long long)b * row_stride * (FP32 ? 4 : 2);
-  MaxSum acc{-INFINITY, 0.f, 0x7fffffff};
-  const int chunks = vocab / EPC;
-  auto take_chunk = [&](const uint4 &w, int c) {
-    const int base = c * EPC;
-    if (FP32) {
-      ms_take(acc, __uint_as_float(w.x), base);
-      ms_take(acc, __uint_as_float(w.y), base + 1);
-      ms_take(acc, __uint_as_float(w.z), base + 2);
-      ms_take(acc, __uint_as_float(w.w), base + 3);
-    } else {
-      ms_take(acc, bf16_lo(w.x), base);
-      ms_take(acc, bf16_hi(w.x), base + 1);
-      ms_take(acc, bf16_lo(w.y), base + 2);
-      ms_take(acc, bf16_hi(w.y), base + 3);
-      ms_take(acc, bf16_lo(w.z), base + 4);
-      ms_take(acc, bf16_hi(w.z), base + 5);
-      ms_take(acc, bf16_lo(w.w), base + 6);
-      ms_take(acc, bf16_hi(w.w), base + 7);
-    }
-  };
-  int c = tid;
-  constexpr int kDeep = 4;                          // 16-byte loads in flight per thread
-  for (; c + (kDeep - 1) * kChainThreads < chunks; c += kDeep * kChainThreads) {
-    uint4 w[kDeep];
-#pragma unroll
-    for (int u = 0; u < kDeep; ++u) w[u] = ld_nc_16(row + (long long)(c + u * kChainThreads) * 16);
-#pragma unroll
-    for (int u = 0; u < kDeep; ++u) take_chunk(w[u], c + u * kChainThreads);
-  }
-  for (; c < chunks; c += kChainThreads) take_chunk(ld_nc_16(row + (long long)c * 16), c);
-  for (int i = chunks * EPC + tid; i < vocab; i += kChainThreads) {     // tail that is no whole chunk
-    const float v = FP32 ? reinterpret_cast<const float *>(row)[i]
-                         : __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(row)[i]);
-    ms_take(acc, v, i);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    MaxSum other;
-    other.m = __shfl_xor_sync(0xffffffffu, acc.m, o);
-    other.s = __shfl_xor_sync(0xffffffffu, acc.s, o);
-    other.i = __shfl_xor_sync(0xffffffffu, acc.i, o);
-    ms_merge(acc, other);
-  }
-  if ((tid & 31) == 0) s_part[tid >> 5] = acc;
-  __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < kChainThreads / 32; ++w) ms_merge(acc, s_part[w]);
-    const float prob = 1.f / acc.s;                 // softmax(row)[token]: the token's logit is the maximum
-    const long long at = (long long)b * t_max + n;
-    parent[at] = n - 1;
-    draft_tok[at] = acc.i;
-    if (tok_prob) tok_prob[at] = prob;
-    n_nodes[b] = n + 1;
-    // n draft tokens now (the root is node 0): stop at delta of them or below the confidence threshold
-    if (n >= max_draft || prob < threshold) active[b] = 0;
-  }
+  const float prob = 1.f / best.s;                  // softmax(row)[token]: the token's logit is the maximum
+  const long long at = (long long)b * t_max + n;
+  parent[at] = n - 1;
+  draft_tok[at] = best.index;
+  if (tok_prob) tok_prob[at] = prob;
+  n_nodes[b] = n + 1;
+  // n draft tokens now (the root is node 0): stop at delta of them or below the confidence threshold
+  if (n >= max_draft || prob < threshold) active[b] = 0;
 }
 
 __global__ void chain_draft_reset_kernel(int *parent, int *draft_tok, float *tok_prob, int *n_nodes, int *active,
                                          int t_max, int batch) {
+  grid_dependency_sync();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx < batch * t_max) {
     parent[idx] = -1;
@@ -140,9 +81,11 @@ extern "C" twig_status chain_draft_reset(int32_t *parent, int32_t *draft_tok, fl
   if (t_max <= 0 || batch <= 0) return TWIG_ERR_SHAPE;
   if (t_max > TWIG_MAX_NODES || batch > TWIG_MAX_BATCH) return TWIG_ERR_UNSUPPORTED;
   const int total = batch * t_max;
-  chain_draft_reset_kernel<<<(total + 255) / 256, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      parent, draft_tok, tok_prob, n_nodes, active, t_max, batch);
-  return launch_status();
+  PdlLaunch L(dim3((total + 255) / 256), dim3(256), 0, static_cast<cudaStream_t>(stream));
+  return cudaLaunchKernelEx(&L.cfg, chain_draft_reset_kernel, parent, draft_tok, tok_prob, n_nodes, active, t_max, batch) ==
+                 cudaSuccess
+             ? TWIG_OK
+             : TWIG_ERR_CUDA;
 }
 
 extern "C" twig_status chain_draft_step(const void *logits, int32_t logits_fp32, int64_t row_stride, int32_t vocab,
@@ -156,20 +99,13 @@ extern "C" twig_status chain_draft_step(const void *logits, int32_t logits_fp32,
   if (!(threshold >= 0.f)) return TWIG_ERR_SHAPE;               // (also refuses NaN)
   const int esz = logits_fp32 ? 4 : 2;
   if (!aligned16(logits) || (row_stride * esz) % 16) return TWIG_ERR_ALIGN;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(batch);
-  cfg.blockDim = dim3(kChainThreads);
-  cfg.stream = static_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = launch_overlap_enabled() ? 1 : 0;
+  const int slices = row_slices(batch, vocab / (16 / esz));
+  ClusterLaunch L(dim3(slices, batch), dim3(kRowThreads), slices, static_cast<cudaStream_t>(stream));
   const long long rs = row_stride;
   const cudaError_t err =
-      logits_fp32 ? cudaLaunchKernelEx(&cfg, chain_draft_step_kernel<true>, logits, rs, vocab, max_draft, threshold, parent,
+      logits_fp32 ? cudaLaunchKernelEx(&L.cfg, chain_draft_step_kernel<true>, logits, rs, vocab, max_draft, threshold, parent,
                                        draft_tok, tok_prob, n_nodes, active, t_max, dev_status)
-                  : cudaLaunchKernelEx(&cfg, chain_draft_step_kernel<false>, logits, rs, vocab, max_draft, threshold, parent,
+                  : cudaLaunchKernelEx(&L.cfg, chain_draft_step_kernel<false>, logits, rs, vocab, max_draft, threshold, parent,
                                        draft_tok, tok_prob, n_nodes, active, t_max, dev_status);
   return err == cudaSuccess ? TWIG_OK : TWIG_ERR_CUDA;
 }

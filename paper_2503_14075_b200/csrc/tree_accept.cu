@@ -3,7 +3,7 @@
 // accepting at each level a child whose token equals its own prediction, and
 // adds one bonus token; the accepted nodes' K/V rows of every layer are then
 // appended to the KV cache (the rejected nodes' rows are simply never copied).
-#include "twig_common.cuh"
+#include "vocab_row.cuh"
 
 namespace twig {
 
@@ -25,31 +25,34 @@ tree_accept_compact_kernel(const int *__restrict__ parent, const int *__restrict
   constexpr int LPR = D / 8;
   __shared__ int s_parent[TWIG_MAX_NODES], s_tok[TWIG_MAX_NODES], s_tgt[TWIG_MAX_NODES];
   __shared__ int s_path[TWIG_MAX_NODES];
-  __shared__ int s_bad, s_best, s_len;
+  __shared__ int s_best;
 
   grid_dependency_sync();
   const int b = blockIdx.y, tid = threadIdx.x;
-  const int n = n_nodes[b];
+  // everything the decision needs is requested at once (one round trip, not four: the kernel is a chain of
+  // them; the one-layer step at batch 1 took 14.3 us of device time, 13.0 with this)
+  const int n = n_nodes[b], base = kv_len[b];
+  int my_parent = -1, my_tok = 0, my_tgt = 0;
+  if (tid < t_max) {
+    my_parent = parent[(long long)b * t_max + tid];
+    my_tok = draft_tok[(long long)b * t_max + tid];
+    my_tgt = base_argmax[(long long)b * t_max + tid];
+  }
   if (n == 0) return;                                   // idle request
   const bool first = blockIdx.x == 0 && tid == 0;
   if (n < 0 || n > t_max) {
     if (first) flag_status(dev_status, b, TWIG_DEV_BAD_TREE);
     return;
   }
-  if (tid == 0) {
-    s_bad = 0;
-    s_best = -1;
-  }
-  __syncthreads();
+  if (tid == 0) s_best = -1;
+  bool bad = false;
   if (tid < n) {
-    const int p = parent[(long long)b * t_max + tid];
-    s_parent[tid] = p;
-    s_tok[tid] = draft_tok[(long long)b * t_max + tid];
-    s_tgt[tid] = base_argmax[(long long)b * t_max + tid];
-    if ((tid == 0) ? (p != -1) : (p < 0 || p >= tid)) s_bad = 1;
+    s_parent[tid] = my_parent;
+    s_tok[tid] = my_tok;
+    s_tgt[tid] = my_tgt;
+    bad = (tid == 0) ? (my_parent != -1) : (my_parent < 0 || my_parent >= tid);
   }
-  __syncthreads();
-  if (s_bad) {
+  if (__syncthreads_or(bad)) {
     if (first) flag_status(dev_status, b, TWIG_DEV_BAD_TREE);
     return;
   }
@@ -69,7 +72,6 @@ tree_accept_compact_kernel(const int *__restrict__ parent, const int *__restrict
   __syncthreads();
   const int alen = s_best / TWIG_MAX_NODES;
   const int winner = TWIG_MAX_NODES - 1 - (s_best % TWIG_MAX_NODES);
-  const int base = kv_len[b];
   if (alen + 1 > d_max || base < 0 || base + alen + 1 > cache.max_len) {
     if (first) flag_status(dev_status, b, alen + 1 > d_max ? TWIG_DEV_BAD_TREE : TWIG_DEV_OVERFLOW);
     return;
@@ -80,7 +82,6 @@ tree_accept_compact_kernel(const int *__restrict__ parent, const int *__restrict
       s_path[j] = x;
       x = s_parent[x];
     }
-    s_len = alen;
   }
   __syncthreads();
   if (blockIdx.x == 0) {
@@ -112,6 +113,10 @@ tree_accept_compact_kernel(const int *__restrict__ parent, const int *__restrict
   }
 
   // every CTA has read kv_len[b] above; the last one to arrive updates it
+  if (gridDim.x == 1) {
+    if (tid == 0) kv_len[b] = base + alen + 1;
+    return;
+  }
   __syncthreads();
   if (tid == 0) {
     __threadfence();
@@ -126,91 +131,34 @@ tree_accept_compact_kernel(const int *__restrict__ parent, const int *__restrict
 
 // ---------------------------------------------------------------------------
 // Greedy target token per tree node: argmax over the vocabulary, lowest index on ties.
-// One CTA per (request, node) row; 16-byte loads, 8 in flight per thread.
+// Grid (slices, nodes, requests), clusters of the slices of a row.
 // ---------------------------------------------------------------------------
-constexpr int kArgmaxThreads = 256;
-
-__device__ __forceinline__ void argmax_take(float v, int i, float &best, int &bi) {
-  if (v > best || (v == best && i < bi)) {
-    best = v;
-    bi = i;
-  }
-}
-
 template <bool FP32>
-__global__ void __launch_bounds__(kArgmaxThreads)
+__global__ void __launch_bounds__(kRowThreads)
 base_argmax_kernel(const void *__restrict__ logits, long long row_stride, int vocab,
                    const int *__restrict__ n_nodes, int t_max, int *__restrict__ out, int *dev_status) {
-  constexpr int EPC = FP32 ? 4 : 8;                 // elements per 16-byte chunk
-  __shared__ float s_v[kArgmaxThreads / 32];
-  __shared__ int s_i[kArgmaxThreads / 32];
+  constexpr int EPC = RowFormat<FP32>::EPC;
+  __shared__ __align__(16) float4 s_peer[kMaxSlices];
+  __shared__ __align__(8) unsigned long long s_bar;
   grid_dependency_sync();
-  const int b = blockIdx.y, node = blockIdx.x, tid = threadIdx.x;
+  const int b = blockIdx.z, node = blockIdx.y, tid = threadIdx.x;
+  SliceMerge sm{s_peer, smem_u32(&s_bar), (int)blockIdx.x, (int)gridDim.x};
   const int n = n_nodes[b];
   if (n < 0 || n > t_max) {
-    if (node == 0 && tid == 0) flag_status(dev_status, b, TWIG_DEV_BAD_TREE);
+    if (node == 0 && sm.rank == 0 && tid == 0) flag_status(dev_status, b, TWIG_DEV_BAD_TREE);
     return;
   }
   if (node >= n) return;
+  sm.start();
   const unsigned char *row = static_cast<const unsigned char *>(logits) +
                              ((long long)b * t_max + node) * row_stride * (FP32 ? 4 : 2);
-  float best = -INFINITY;
-  int bi = 0x7fffffff;
-  const int chunks = vocab / EPC;
-  auto take_chunk = [&](const uint4 &w, int c) {
-    const int base = c * EPC;
-    if (FP32) {
-      argmax_take(__uint_as_float(w.x), base, best, bi);
-      argmax_take(__uint_as_float(w.y), base + 1, best, bi);
-      argmax_take(__uint_as_float(w.z), base + 2, best, bi);
-      argmax_take(__uint_as_float(w.w), base + 3, best, bi);
-    } else {
-      argmax_take(bf16_lo(w.x), base, best, bi);
-      argmax_take(bf16_hi(w.x), base + 1, best, bi);
-      argmax_take(bf16_lo(w.y), base + 2, best, bi);
-      argmax_take(bf16_hi(w.y), base + 3, best, bi);
-      argmax_take(bf16_lo(w.z), base + 4, best, bi);
-      argmax_take(bf16_hi(w.z), base + 5, best, bi);
-      argmax_take(bf16_lo(w.w), base + 6, best, bi);
-      argmax_take(bf16_hi(w.w), base + 7, best, bi);
-    }
-  };
-  constexpr int kDeep = 8;                          // 16-byte loads in flight per thread
-  // (every batch is predicated, so that a row that is no multiple of the batch never falls back to one
-  // load per round trip)
-  for (int c0 = tid; c0 < chunks; c0 += kDeep * kArgmaxThreads) {
-    uint4 w[kDeep];
-#pragma unroll
-    for (int u = 0; u < kDeep; ++u) {
-      const int c = c0 + u * kArgmaxThreads;
-      if (c < chunks) w[u] = ld_nc_16(row + (long long)c * 16);
-    }
-#pragma unroll
-    for (int u = 0; u < kDeep; ++u) {
-      const int c = c0 + u * kArgmaxThreads;
-      if (c < chunks) take_chunk(w[u], c);
-    }
-  }
-  for (int i = chunks * EPC + tid; i < vocab; i += kArgmaxThreads) {     // tail that is no whole chunk
-    const float v = FP32 ? reinterpret_cast<const float *>(row)[i]
-                         : __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(row)[i]);
-    argmax_take(v, i, best, bi);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, best, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    argmax_take(ov, oi, best, bi);
-  }
-  if ((tid & 31) == 0) {
-    s_v[tid >> 5] = best;
-    s_i[tid >> 5] = bi;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < kArgmaxThreads / 32; ++w) argmax_take(s_v[w], s_i[w], best, bi);
-    out[(long long)b * t_max + node] = bi;
-  }
+  const int chunks = vocab / EPC, per = (chunks + sm.slices - 1) / sm.slices;
+  RowBest best = scan_slice<FP32, false>(row, sm.rank * per, min(chunks, (sm.rank + 1) * per),
+                                         sm.rank == 0 && chunks * EPC < vocab, vocab);
+  const bool landed = sm.merge<false>(best);
+  if (sm.rank > 0 || tid != 0) return;
+  if (landed) out[(long long)b * t_max + node] = best.index;
+  else flag_status(dev_status, b, TWIG_DEV_INTERNAL);
 }
 
 }  // namespace twig
@@ -226,19 +174,12 @@ extern "C" twig_status tree_base_argmax(const void *logits, int32_t logits_fp32,
   if (t_max > TWIG_MAX_NODES || batch > TWIG_MAX_BATCH) return TWIG_ERR_UNSUPPORTED;
   const int esz = logits_fp32 ? 4 : 2;
   if (!aligned16(logits) || (row_stride * esz) % 16) return TWIG_ERR_ALIGN;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(t_max, batch);
-  cfg.blockDim = dim3(kArgmaxThreads);
-  cfg.stream = static_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = launch_overlap_enabled() ? 1 : 0;
+  const int slices = row_slices((long long)t_max * batch, vocab / (16 / esz));
+  ClusterLaunch L(dim3(slices, t_max, batch), dim3(kRowThreads), slices, static_cast<cudaStream_t>(stream));
   const long long rs = row_stride;
   const cudaError_t err =
-      logits_fp32 ? cudaLaunchKernelEx(&cfg, base_argmax_kernel<true>, logits, rs, vocab, n_nodes, t_max, base_argmax, dev_status)
-                  : cudaLaunchKernelEx(&cfg, base_argmax_kernel<false>, logits, rs, vocab, n_nodes, t_max, base_argmax, dev_status);
+      logits_fp32 ? cudaLaunchKernelEx(&L.cfg, base_argmax_kernel<true>, logits, rs, vocab, n_nodes, t_max, base_argmax, dev_status)
+                  : cudaLaunchKernelEx(&L.cfg, base_argmax_kernel<false>, logits, rs, vocab, n_nodes, t_max, base_argmax, dev_status);
   return err == cudaSuccess ? TWIG_OK : TWIG_ERR_CUDA;
 }
 

@@ -91,6 +91,26 @@ struct PdlLaunch {
   }
 };
 
+// The same with clusters of `cluster` CTAs along x.
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  ClusterLaunch(dim3 grid, dim3 block, int cluster, cudaStream_t st, size_t smem = 0) {
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = launch_overlap_enabled() ? 2 : 1;
+  }
+};
+
 inline twig_status launch_status() {
   return cudaGetLastError() == cudaSuccess ? TWIG_OK : TWIG_ERR_CUDA;
 }
