@@ -138,11 +138,6 @@ ttp_logits_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__re
 // (slices, batch), any CTA size, every CTA takes a slice of the request's visual tokens (the
 // per-head statistics are merged from the logits stage's per-warp partials by every CTA: cheap).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t order_key(float x) {
-  const uint32_t u = __float_as_uint(x);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
 // exclusive block scan of `x` over 1024 threads; returns the block total in `total`
 __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t *warp_sums, uint32_t &total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

@@ -142,6 +142,12 @@ __device__ __forceinline__ void st_16(void *p, const uint4 &r) {
                : "memory");
 }
 
+// unsigned integers in the order of the floats
+__device__ __forceinline__ uint32_t order_key(float x) {
+  const uint32_t u = __float_as_uint(x);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 #endif
