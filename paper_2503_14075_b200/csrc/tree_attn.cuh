@@ -98,6 +98,9 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
+__device__ __forceinline__ void st_cluster_u32(uint32_t dst, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(dst), "r"(v) : "memory");
+}
 // stores into a cluster CTA's shared memory (this CTA's own included); that CTA's mbarrier
 // counts the bytes once they have landed
 __device__ __forceinline__ void st_async_b32x2(uint32_t dst, uint32_t a, uint32_t b, uint32_t bar) {

@@ -6,7 +6,7 @@
 // over heads).  TopR is Eq. 3's selection with the lower index winning ties
 // and sequence order kept.  The gather applies the pruned token list to the
 // cached K/V rows of every layer; position ids travel with their rows.
-#include "twig_common.cuh"
+#include "tree_attn.cuh"
 
 namespace twig {
 
@@ -15,7 +15,7 @@ constexpr int kScoreKeysPerCta = 128;
 constexpr int kScoreWarps = kScoreThreads / 32;   // every warp of the logits stage writes one partial (max, sum) per head
 constexpr int kMaxGroup = 16;   // query heads per kv head
 constexpr int kMaxQHeads = 128;
-constexpr int kTopkThreads = 1024;
+constexpr int kTopkThreads = 512;
 
 // per-request layout check shared by the three stages
 __device__ __forceinline__ bool layout_ok(int lp, int vs, int nv, int k_max_len, int m_max) {
@@ -131,14 +131,7 @@ ttp_logits_kernel(const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__re
   }
 }
 
-// ---------------------------------------------------------------------------
-// Stage 1b + 2: softmax per head, mean over heads -> scores; then exact TopR.
-// mode bit 0: compute scores from the logits; bit 1: select.  Without bit 0 the scores are read from
-// `scores`.  With the selection: one CTA of 1024 threads per request.  Scores alone: grid
-// (slices, batch), any CTA size, every CTA takes a slice of the request's visual tokens (the
-// per-head statistics are merged from the logits stage's per-warp partials by every CTA: cheap).
-// ---------------------------------------------------------------------------
-// exclusive block scan of `x` over 1024 threads; returns the block total in `total`
+// exclusive block scan of `x` over the CTA; returns the block total in `total`
 __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t *warp_sums, uint32_t &total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t inc = x;
@@ -150,21 +143,35 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t *w
   if (lane == 31) warp_sums[warp] = inc;
   __syncthreads();
   if (warp == 0) {
-    uint32_t w = warp_sums[lane], winc = w;
+    uint32_t w = lane < kTopkThreads / 32 ? warp_sums[lane] : 0u, winc = w;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, winc, o);
       if (lane >= o) winc += y;
     }
-    warp_sums[lane] = winc - w;
-    if (lane == 31) warp_sums[32] = winc;
+    if (lane < kTopkThreads / 32) warp_sums[lane] = winc - w;
+    if (lane == 31) warp_sums[kTopkThreads / 32] = winc;
   }
   __syncthreads();
   const uint32_t res = warp_sums[warp] + inc - x;
-  total = warp_sums[32];
+  total = warp_sums[kTopkThreads / 32];
   __syncthreads();
   return res;
 }
+
+// ---------------------------------------------------------------------------
+// Stage 1b + 2: softmax per head, mean over heads -> scores; then exact TopR.
+// mode bit 0: compute scores from the logits; bit 1: select.  Without bit 0 the scores are read from
+// `scores`.  Grid (slices, batch): every CTA computes the scores of a slice of the request's visual tokens (the
+// per-head statistics are merged from the logits stage's per-warp partials by every CTA: cheap).  With the
+// selection the slices of a request are a cluster; the ordered keys meet in the first CTA's shared memory
+// (DSMEM), which selects.
+// What bounds it is latency: one CTA of 1024 threads per request took 14.5 us (576 tokens, 32 heads) to
+// 19 us (2880 tokens), four radix passes of histogram atomics and scans among it.  The R-th largest key
+// is now found bit by bit from the first bit in which the keys differ, one count and one barrier a bit,
+// and usually ends early, when exactly R keys reach the value.
+// ---------------------------------------------------------------------------
+constexpr int kTopkKeys = 8;         // keys a thread holds in registers (4096 tokens; beyond, they are read again)
 
 __global__ void __launch_bounds__(kTopkThreads)
 ttp_finalize_topk_kernel(const float *__restrict__ logits, int lstride, const float2 *__restrict__ stats,
@@ -173,27 +180,31 @@ ttp_finalize_topk_kernel(const float *__restrict__ logits, int lstride, const fl
                          const int *__restrict__ n_vis, const int *__restrict__ keep, int norm_scope,
                          float *__restrict__ scores, int m_max, int *__restrict__ kept_idx, int r_max,
                          int *dev_status, int mode) {
-  extern __shared__ uint32_t keys[];                 // [m_max] fp32 scores, then ordered keys
+  extern __shared__ uint32_t keys[];                 // [m_max] ordered keys (first CTA of a request)
   __shared__ float h_max[kMaxQHeads], h_inv[kMaxQHeads];
-  __shared__ uint32_t hist[256];
-  __shared__ uint32_t warp_sums[33];
-  __shared__ uint32_t sel_digit, sel_remaining;
+  constexpr int kWarps = kTopkThreads / 32;
+  __shared__ uint32_t s_low[kWarps], s_high[kWarps], s_count[2][kWarps];
+  __shared__ uint32_t s_bits[TWIG_MAX_VISUAL / 32];
+  __shared__ uint32_t warp_sums[kWarps + 1];
 
   // the kernel after this one (the gather of the fused call) may start on what does not depend on the
   // selection; this kernel itself reads its predecessor's output from here on
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nt = blockDim.x;
+  const int slice = blockIdx.x, slices = gridDim.x;
+  constexpr int nt = kTopkThreads;
   const int nv = n_vis[b];
   float *sc = scores + (long long)b * m_max;
+  const bool meet = (mode & 2) && slices > 1;        // (uniform over the cluster, like every exit before the barrier)
 
   if (mode & 1) {
     const int lp = prefix_len[b], vs = vis_start[b];
     if (!layout_ok(lp, vs, nv, k_max_len, m_max)) {
-      if (tid == 0 && blockIdx.x == 0) flag_status(dev_status, b, TWIG_DEV_BAD_LAYOUT);
+      if (tid == 0 && slice == 0) flag_status(dev_status, b, TWIG_DEV_BAD_LAYOUT);
       return;
     }
+    if (meet) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");    // this CTA is running
     const int lo = norm_scope ? vs : 0, hi = norm_scope ? vs + nv : lp;
     // partials of the logits stage that may hold keys of the scope: those of its chunks (none for an
     // empty scope); a partial without a key in scope is (-inf, 0)
@@ -239,8 +250,9 @@ ttp_finalize_topk_kernel(const float *__restrict__ logits, int lstride, const fl
       }
     }
     __syncthreads();
+    if (meet) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // the first CTA is running
     const float inv_h = 1.f / (float)n_q_heads;
-    for (int m = blockIdx.x * nt + tid; m < m_max; m += gridDim.x * nt) {
+    for (int m = slice * nt + tid; m < m_max; m += slices * nt) {
       float acc = 0.f;
       if (m < nv) {
         const float *z = logits + (long long)b * n_q_heads * lstride + vs + m;
@@ -263,89 +275,112 @@ ttp_finalize_topk_kernel(const float *__restrict__ logits, int lstride, const fl
         acc *= inv_h;
       }
       sc[m] = acc;
-      if (mode & 2) keys[m] = order_key(acc);
+      if ((mode & 2) && m < nv) {
+        if (slice == 0) keys[m] = order_key(acc);
+        else st_cluster_u32(map_to_cta(smem_u32(keys + m), 0), order_key(acc));
+      }
     }
   } else {
     if (nv < 0 || nv > m_max) {
       if (tid == 0) flag_status(dev_status, b, TWIG_DEV_BAD_LAYOUT);
       return;
     }
-    for (int m = tid; m < nv; m += kTopkThreads) keys[m] = order_key(sc[m]);
+    for (int m = tid; m < nv; m += nt) keys[m] = order_key(sc[m]);
   }
   if (!(mode & 2)) return;
+  if (meet) {                                        // the other slices' keys have arrived
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (slice > 0) return;
+  } else {
+    __syncthreads();
+  }
   const int R = keep[b];
   if (R < 0 || R > nv || R > r_max) {
     if (tid == 0) flag_status(dev_status, b, TWIG_DEV_BAD_KEEP);
     return;
   }
   int *out = kept_idx + (long long)b * r_max;
-  for (int i = R + tid; i < r_max; i += kTopkThreads) out[i] = -1;
+  for (int i = R + tid; i < r_max; i += nt) out[i] = -1;
   if (R == 0) return;
-  __syncthreads();
 
-  // radix select, 8 bits per pass from the top: the R-th largest key
-  uint32_t prefix = 0, mask = 0;
-  uint32_t remaining = (uint32_t)R;
+  // this thread's keys: tokens tid, tid + nt, .. (0, which no score has, past the last one)
+  const int rounds = (nv + nt - 1) / nt;
+  uint32_t key[kTopkKeys], low = 0xffffffffu, high = 0;
+#pragma unroll
+  for (int q = 0; q < kTopkKeys; ++q) key[q] = tid + q * nt < nv ? keys[tid + q * nt] : 0u;
+  auto each_key = [&](auto &&f) {
+#pragma unroll
+    for (int q = 0; q < kTopkKeys; ++q)
+      if (q < rounds) f(key[q]);
 #pragma unroll 1
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    if (tid < 256) hist[tid] = 0;
+    for (int m = tid + kTopkKeys * nt; m < nv; m += nt) f(keys[m]);
+  };
+  each_key([&](uint32_t k) {
+    low = min(low, k != 0u ? k : 0xffffffffu);
+    high = max(high, k);
+  });
+  auto count = [&](auto &&pred, int parity) {        // keys of the request for which pred holds
+    uint32_t c = 0;
+    each_key([&](uint32_t k) { c += pred(k) ? 1u : 0u; });
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) s_count[parity][warp] = c;
     __syncthreads();
-    // (scores of one request are close to each other, so in the top passes nearly all keys share a
-    // digit: the lanes of a warp that hold the same digit add their count with one atomic)
-    for (int base = 0; base < nv; base += kTopkThreads) {
-      const int m = base + tid;
-      const uint32_t key = m < nv ? keys[m] : 0u;
-      const bool cand = m < nv && (key & mask) == prefix;
-      const uint32_t digit = cand ? (key >> shift) & 255u : 256u + (uint32_t)lane;     // non-candidates match nobody
-      const unsigned peers = __match_any_sync(0xffffffffu, digit);
-      if (cand && lane == __ffs(peers) - 1) atomicAdd(&hist[digit], (uint32_t)__popc(peers));
-    }
-    __syncthreads();
-    if (warp == 0) {
-      uint32_t c[8], mine = 0;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        c[i] = hist[lane * 8 + i];
-        mine += c[i];
-      }
-      uint32_t suf = mine;   // inclusive suffix sum over lanes (lane 31 = top digits)
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_down_sync(0xffffffffu, suf, o);
-        if (lane + o < 32) suf += y;
-      }
-      uint32_t above = suf - mine;
-      if (above < remaining && remaining <= suf) {
-#pragma unroll
-        for (int i = 7; i >= 0; --i) {
-          if (above < remaining && remaining <= above + c[i]) {
-            sel_digit = lane * 8 + i;
-            sel_remaining = remaining - above;
-          }
-          above += c[i];
-        }
-      }
-    }
-    __syncthreads();
-    prefix |= sel_digit << shift;
-    mask |= 255u << shift;
-    remaining = sel_remaining;
-    __syncthreads();
+    return __reduce_add_sync(0xffffffffu, lane < kWarps ? s_count[parity][lane] : 0u);
+  };
+  low = __reduce_min_sync(0xffffffffu, low);
+  high = __reduce_max_sync(0xffffffffu, high);
+  if (lane == 0) {
+    s_low[warp] = low;
+    s_high[warp] = high;
   }
-  const uint32_t tau = prefix, need_eq = remaining;
+  __syncthreads();
+  low = __reduce_min_sync(0xffffffffu, lane < kWarps ? s_low[lane] : 0xffffffffu);
+  high = __reduce_max_sync(0xffffffffu, lane < kWarps ? s_high[lane] : 0u);
+  // tau: the R-th largest key, or a value that exactly R keys reach
+  uint32_t bit = low == high ? 0u : 0x80000000u >> __clz(low ^ high);
+  uint32_t tau = bit == 0 ? low : low & ~(2 * bit - 1), reach = (uint32_t)nv;
+  int parity = 0;
+#pragma unroll 1
+  for (; bit != 0 && reach != (uint32_t)R; bit >>= 1, parity ^= 1) {
+    const uint32_t t = tau | bit, c = count([t](uint32_t k) { return k >= t; }, parity);
+    if (c >= (uint32_t)R) {
+      tau = t;
+      reach = c;
+    }
+  }
+  // more than R only with equal keys at tau: the lowest indices of them
+  uint32_t need_eq = 0;
+  if (reach > (uint32_t)R) {
+    const uint32_t t = tau;
+    need_eq = count([t](uint32_t k) { return k == t; }, parity) - (reach - (uint32_t)R);
+    parity ^= 1;
+  }
 
-  // ordered compaction: keys above tau, plus the first need_eq keys equal to tau
-  uint32_t run_gt = 0, run_eq = 0;
-  for (int base = 0; base < nv; base += kTopkThreads) {
-    const int m = base + tid;
-    const uint32_t key = (m < nv) ? keys[m] : 0u;
-    const uint32_t gt = (m < nv && key > tau), eq = (m < nv && key == tau);
-    uint32_t total;
-    const uint32_t ex = block_exclusive_scan(gt | (eq << 16), warp_sums, total);
-    const uint32_t gt_before = run_gt + (ex & 0xffffu), eq_before = run_eq + (ex >> 16);
-    if (gt || (eq && eq_before < need_eq)) out[gt_before + min(eq_before, need_eq)] = m;
-    run_gt += total & 0xffffu;
-    run_eq += total >> 16;
+  // ordered compaction: one bit per token, then the tokens before each word of bits
+  uint32_t run_eq = 0;
+#pragma unroll 1
+  for (int q = 0; q < rounds; ++q) {
+    const int m = q * nt + tid;
+    const uint32_t k = m < nv ? keys[m] : 0u;
+    bool kept = m < nv && k >= tau;
+    if (reach > (uint32_t)R) {
+      const bool eq = m < nv && k == tau;
+      uint32_t total;
+      const uint32_t before = run_eq + block_exclusive_scan(eq ? 1u : 0u, warp_sums, total);
+      if (eq) kept = before < need_eq;
+      run_eq += total;
+    }
+    const unsigned bits = __ballot_sync(0xffffffffu, kept);
+    if (lane == 0) s_bits[q * kWarps + warp] = bits;
+  }
+  __syncthreads();
+  const int words = rounds * kWarps;                 // at most kTopkThreads
+  uint32_t total;
+  const uint32_t at = block_exclusive_scan(tid < words ? (uint32_t)__popc(s_bits[tid]) : 0u, warp_sums, total);
+  if (tid < words) {
+    uint32_t bits = s_bits[tid], pos = at;
+    for (; bits; bits &= bits - 1) out[pos++] = tid * 32 + __ffs(bits) - 1;
   }
 }
 
@@ -696,10 +731,10 @@ static twig_status launch_finalize(const float *logits, const ScoreArgs &a, cons
       return TWIG_ERR_CUDA;
     attr_set = true;
   }
-  // the selection needs a request's scores in one CTA; scores alone are spread over slices of 256 tokens
-  constexpr int kSliceThreads = 256;
-  const dim3 grid = select ? dim3(1, a.batch) : dim3((a.m_max + kSliceThreads - 1) / kSliceThreads, a.batch);
-  PdlLaunch L(grid, dim3(select ? kTopkThreads : kSliceThreads), smem, st);
+  // slices of a CTA's tokens; with the selection they are a cluster (of at most eight CTAs)
+  int slices = (mode & 1) ? (a.m_max + kTopkThreads - 1) / kTopkThreads : 1;
+  if (select) slices = slices > 4 ? 8 : slices > 2 ? 4 : slices;
+  ClusterLaunch L(dim3(slices, a.batch), dim3(kTopkThreads), select ? slices : 1, st, smem);
   const int ls = logits_stride(a.k_max_len);
   const float2 *stats = logits ? reinterpret_cast<const float2 *>(reinterpret_cast<const unsigned char *>(logits) +
                                                                   logits_bytes(a.batch, a.n_q_heads, a.k_max_len))
