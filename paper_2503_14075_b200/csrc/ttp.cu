@@ -196,7 +196,7 @@ ttp_finalize_topk_kernel(const float *__restrict__ logits, int lstride, const fl
   __shared__ float h_max[kMaxQHeads], h_inv[kMaxQHeads];
   constexpr int kWarps = kTopkThreads / 32;
   __shared__ uint32_t s_low[kWarps], s_high[kWarps], s_count[2][kWarps];
-  __shared__ uint32_t s_bits[TWIG_MAX_VISUAL / 32];
+  __shared__ uint32_t s_bits[TWIG_MAX_VISUAL / 32], s_before[TWIG_MAX_VISUAL / 32];
   __shared__ uint32_t warp_sums[kWarps + 1];
 
   // the kernel after this one (the gather of the fused call) may start on what does not depend on the
@@ -206,7 +206,7 @@ ttp_finalize_topk_kernel(const float *__restrict__ logits, int lstride, const fl
   const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int slice = blockIdx.x, slices = gridDim.x;
   constexpr int nt = kTopkThreads;
-  const int nv = n_vis[b];
+  const int nv = n_vis[b], R = (mode & 2) ? keep[b] : 0;
   float *sc = scores + (long long)b * m_max;
   const bool meet = (mode & 2) && slices > 1;        // (uniform over the cluster, like every exit before the barrier)
 
@@ -218,6 +218,12 @@ ttp_finalize_topk_kernel(const float *__restrict__ logits, int lstride, const fl
     }
     if (meet) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");    // this CTA is running
     const int lo = norm_scope ? vs : 0, hi = norm_scope ? vs + nv : lp;
+    // the logits of this thread's first token are requested with the statistics (32 heads: one round trip)
+    const int m0 = slice * nt + tid;
+    const float *z0 = logits + (long long)b * n_q_heads * lstride + vs + m0;
+    float ahead[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) ahead[i] = m0 < nv && i < n_q_heads ? z0[(long long)i * lstride] : 0.f;
     // partials of the logits stage that may hold keys of the scope: those of its chunks (none for an
     // empty scope); a partial without a key in scope is (-inf, 0)
     const int c_lo = lo / kScoreKeysPerCta, c_hi = hi > lo ? (hi - 1) / kScoreKeysPerCta : c_lo - 1;
@@ -272,7 +278,7 @@ ttp_finalize_topk_kernel(const float *__restrict__ logits, int lstride, const fl
         for (; h + 32 <= n_q_heads; h += 32) {         // 32 heads' logits in flight: one round trip
           float zz[32];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) zz[i] = z[(long long)(h + i) * lstride];
+          for (int i = 0; i < 32; ++i) zz[i] = m == m0 && h == 0 ? ahead[i] : z[(long long)(h + i) * lstride];
 #pragma unroll
           for (int i = 0; i < 32; ++i) acc += expf(zz[i] - h_max[h + i]) * h_inv[h + i];
         }
@@ -307,7 +313,6 @@ ttp_finalize_topk_kernel(const float *__restrict__ logits, int lstride, const fl
   } else {
     __syncthreads();
   }
-  const int R = keep[b];
   if (R < 0 || R > nv || R > r_max) {
     if (tid == 0) flag_status(dev_status, b, TWIG_DEV_BAD_KEEP);
     return;
@@ -390,9 +395,12 @@ ttp_finalize_topk_kernel(const float *__restrict__ logits, int lstride, const fl
   const int words = rounds * kWarps;                 // at most kTopkThreads
   uint32_t total;
   const uint32_t at = block_exclusive_scan(tid < words ? (uint32_t)__popc(s_bits[tid]) : 0u, warp_sums, total);
-  if (tid < words) {
-    uint32_t bits = s_bits[tid], pos = at;
-    for (; bits; bits &= bits - 1) out[pos++] = tid * 32 + __ffs(bits) - 1;
+  if (tid < words) s_before[tid] = at;
+  __syncthreads();
+#pragma unroll 1
+  for (int q = 0; q < rounds; ++q) {
+    const uint32_t bits = s_bits[q * kWarps + warp];
+    if ((bits >> lane) & 1u) out[s_before[q * kWarps + warp] + __popc(bits & ((1u << lane) - 1u))] = q * nt + tid;
   }
 }
 
