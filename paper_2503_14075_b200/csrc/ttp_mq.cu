@@ -2,8 +2,9 @@
 // every visual token, summed over those tokens and averaged over heads,
 //   a[m] = (1/H) sum_h sum_i softmax_{j <= t_i}(q_i . k_j / sqrt(d))[vis_start + m],
 // t_i = vis_start + n_vis + i the prompt position of text token i.  Unlike the single-query score
-// this is an N x L attention-map reduction.  Three kernels, each launched so that it may be
-// scheduled while its predecessor drains:
+// this is an N x L attention-map reduction.  Small calls (see ttp_mq_held_kernel and the rule in
+// ttp_score_multiquery) keep the logits in tensor memory and make one pass plus the sum of step 3; the others
+// run three kernels, each launched so that it may be scheduled while its predecessor drains:
 //   1. probabilities: a CTA takes 64 query rows of one head and a run of kChunk-key chunks.  Q (cp.async)
 //      and the key tiles (TMA) go to shared memory in the 128-byte-swizzled layout of the matrix
 //      descriptors, one thread issues S = Q K^T per chunk (tcgen05.mma, M = 64, N = kChunk, fp32 in
@@ -22,7 +23,7 @@
 #include <mutex>
 #include <type_traits>
 
-#include "tcgen05_common.cuh"
+#include "columns.cuh"
 
 namespace twig {
 
@@ -67,10 +68,300 @@ inline size_t mq_probs_bytes(size_t items, int n_chunks) { return items * n_chun
 inline size_t mq_stats_bytes(size_t items, int n_chunks) { return items * 2 * n_chunks * kMqRows * sizeof(float2); }
 inline size_t mq_partial_bytes(size_t items, int m_max) { return ((items * m_max * sizeof(float)) + 15) & ~(size_t)15; }
 
-// ---- 1. probabilities and per-chunk statistics ----
+
+// ---- up to 4096 keys: one pass, nothing but column sums leaves the chip ----
+// grid (cluster, heads * n_row_blocks, batch): a cluster takes one item (request, head, block of 64 text rows), its
+// CTAs an equal share of the item's 128-key chunks, at most kHeld each.  The products are transposed,
+// S^T = K Q^T (tcgen05, M = 128 keys, N = 64 rows), and every chunk has 64 columns of tensor memory of its
+// own, so the logits stay where they are until the rows' denominators are known:
+//   pass A, chunk by chunk as the keys arrive: row sums of exponentials relative to a reference (a key per
+//     thread, half of the rows each: sums stay in registers, the reference is checked, not reduced);
+//   the CTAs exchange (reference, sum) of the 64 rows through distributed shared memory;
+//   pass B: a visual key's score is the sum over the rows of exp2(logit - reference - log2 sum): one multiply-add
+//     and one exponential per element, the sum over rows in the thread.
+// Bound by the latency of its chain (tile, product, two passes, one exchange).  One prompt of 3008 keys, 64 text
+// rows and 32 heads: 17.6 us; the three kernels below, each with a ramp of its own and 2 bytes per (row, key)
+// written and read between them, 23.7.  4 heads and 100 visual tokens: 8.0 and 16.5 us.
+constexpr int kHeld = 4;             // chunks of a CTA: 256 columns, so that two CTAs share an SM
+constexpr int kHeldBufs = 2;         // key tiles (a tile is free as soon as its product has read it)
+constexpr int kHeldThreads = 320;    // warps 0-7: rows and columns; 8: tiles; 9: products
+constexpr float kHeldLazy = 60.f;    // raise a row's reference only beyond this (log2 units; the sums are fp32)
+
+template <int D>
+constexpr int held_smem() { return kMqRows * D * 2 + kHeldBufs * kChunk * D * 2 + 8 * kMqRows * 8 + kHeld * kChunk * 4; }
+
+template <int D>
+__global__ void __launch_bounds__(kHeldThreads, 2)
+ttp_mq_held_kernel(const __nv_bfloat16 *__restrict__ q_text, int n_text_max, const __grid_constant__ CUtensorMap kmap,
+                   int k_max_len, const int *__restrict__ prefix_len, const int *__restrict__ vis_start,
+                   const int *__restrict__ n_vis, int n_q_heads, int group, float sc, int n_row_blocks,
+                   float *__restrict__ partial, int m_max, int *dev_status) {
+  constexpr int CPR = D / 8, R = kMqRows, RH = R / 2;
+  constexpr int Q_BYTES = R * D * 2, K_BYTES = kChunk * D * 2;
+  extern __shared__ __align__(1024) unsigned char smem[];   // Q | key tiles | peers' (reference, sum) | column sums
+  __shared__ __align__(16) float s_red[4 * R], s_m[R], s_c[R];
+  // full[bufs], empty[bufs], ready[kHeld], q, recv
+  __shared__ __align__(8) unsigned long long s_bar[2 * kHeldBufs + kHeld + 2];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // (uniform for the compiler too: see umma8_kk)
+  const int rank = blockIdx.x, n_ctas = gridDim.x;
+  const int h = blockIdx.y / n_row_blocks, qb = blockIdx.y % n_row_blocks, b = blockIdx.z;
+  grid_dependency_sync();
+  const MqLayout y = mq_layout(prefix_len, vis_start, n_vis, b, k_max_len, m_max, n_text_max);
+  if (!y.ok) {
+    if (tid == 0 && rank == 0 && blockIdx.y == 0) flag_status(dev_status, b, TWIG_DEV_BAD_LAYOUT);
+    return;
+  }
+  const int row0 = qb * R;
+  if (row0 >= y.n_text || y.nv == 0) return;          // (every exit so far is uniform over the cluster)
+  const int rows = min(R, y.n_text - row0);
+  const int t_first = y.vs + y.nv + row0;             // prompt position of this block's first query
+  const int n_c = (t_first + rows - 1) / kChunk + 1;  // chunks that hold a key some row sees
+  const int per = (n_c + n_ctas - 1) / n_ctas;        // (at most kHeld: the host sized the cluster)
+  const int c_begin = min(n_c, rank * per), n_it = min(n_c, c_begin + per) - c_begin;
+
+  const uint32_t bars = smem_u32(s_bar);
+  auto bar_full = [&](int i) { return bars + 8 * i; };
+  auto bar_empty = [&](int i) { return bars + 8 * (kHeldBufs + i); };
+  auto bar_ready = [&](int i) { return bars + 8 * (2 * kHeldBufs + i); };
+  const uint32_t bar_q = bars + 8 * (2 * kHeldBufs + kHeld), bar_recv = bar_q + 8;
+  const uint32_t q_s = smem_u32(smem), k_s = q_s + Q_BYTES;
+  float2 *peer = reinterpret_cast<float2 *>(smem + Q_BYTES + kHeldBufs * K_BYTES);        // [CTA][row]
+  float *colsum = reinterpret_cast<float *>(peer + 8 * R);                                // [chunk][key]: the second half's sums
+  auto load_tile = [&](int it) {                      // (one thread)
+    const int buf = it % kHeldBufs;
+    mbar_arrive_expect_tx(bar_full(buf), K_BYTES);
+#pragma unroll
+    for (int p = 0; p < D / 64; ++p)
+      tma_load_4d(k_s + buf * K_BYTES + p * kChunk * 128, &kmap, bar_full(buf), p * 64, (c_begin + it) * kChunk, h / group, b);
+  };
+  if (tid == 256) {                                   // the first tiles are on their way before anything else is ready
+    for (int i = 0; i < kHeldBufs; ++i) {
+      mbar_init(bar_full(i), 1);
+      mbar_init(bar_empty(i), 1);
+    }
+    mbar_init_fence_cluster();
+    fence_async_smem();
+    for (int it = 0; it < kHeldBufs && it < n_it; ++it) load_tile(it);
+  }
+  if (warp < 8) {                                     // Q (zero rows past the last)
+    const __nv_bfloat16 *qsrc = q_text + (((long long)b * n_q_heads + h) * n_text_max + row0) * D;
+#pragma unroll
+    for (int cid = tid; cid < R * CPR; cid += 256) {
+      const int r = cid / CPR, cc = cid % CPR;
+      cp_async_16(q_s + mq_off(r, cc, R), qsrc + (long long)(r < rows ? r : 0) * D + cc * 8, r < rows);
+    }
+    cp_async_commit();
+  }
+  if (tid == 0) {
+    s_fail = 0;
+    for (int i = 0; i < kHeld; ++i) mbar_init(bar_ready(i), 1);
+    mbar_init(bar_q, 8);
+    mbar_init(bar_recv, 1);
+    if (n_ctas > 1) mbar_arrive_expect_tx(bar_recv, (uint32_t)(n_ctas - 1) * R * 8);
+    mbar_init_fence_cluster();
+  }
+  if (warp == 9) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(kHeld * R) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (n_ctas > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");    // this CTA's barrier is set up
+  const uint32_t tmem = s_tmem;
+  volatile int *fail = &s_fail;
+  const int quad = warp & 3, half = (warp >> 2) & 1, h0 = half * RH;
+  const uint32_t t_lane = tmem + ((uint32_t)(quad * 32) << 16) + h0;
+  const int kl = quad * 32 + lane;                    // this thread's key within a chunk
+  float l[RH];
+
+  if (warp == 8) {
+    // ================= key tiles =================
+    const uint32_t leader = elect_one();
+    bool ok = true;
+    for (int it = kHeldBufs; it < n_it && ok; ++it) {
+      ok = mbar_wait(bar_empty(it % kHeldBufs), (it / kHeldBufs - 1) & 1, fail);
+      if (ok && leader) load_tile(it);
+    }
+    if (!ok && lane == 0) s_fail = 1;
+  } else if (warp == 9) {
+    // ================= products =================
+    const uint32_t leader = elect_one();
+    constexpr uint32_t kIdesc = instr_desc(kChunk, R, false);
+    bool ok = n_it == 0 || mbar_wait(bar_q, 0, fail);
+    for (int it = 0; it < n_it && ok; ++it) {
+      const int buf = it % kHeldBufs;
+      ok = mbar_wait(bar_full(buf), (it / kHeldBufs) & 1, fail);
+      if (!ok) break;
+      const uint64_t kd = smem_desc(k_s + buf * K_BYTES, 16), qd = smem_desc(q_s, 16);
+      if constexpr (D == 128) {
+        umma8_kk<kChunk * 128, R * 128>(leader, tmem + it * R, kd, qd, kIdesc);
+      } else {
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks)
+          if (leader) umma(tmem + it * R, kd + 2 * ks, qd + 2 * ks, kIdesc, ks > 0);
+      }
+      umma_commit_if(leader, bar_ready(it));
+      umma_commit_if(leader, bar_empty(buf));
+    }
+    if (!ok && lane == 0) s_fail = 1;
+  } else {
+    // ================= rows (no wait below is followed by a break: the warps meet at every barrier) =================
+    cp_async_wait<0>();
+    fence_async_smem();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar_q);
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < RH; ++i) l[i] = 0.f;
+    for (int it = 0; it < n_it; ++it) {
+      const int j = (c_begin + it) * kChunk + kl;
+      const bool edge = (c_begin + it) * kChunk + kChunk - 1 > t_first;      // (uniform) some key is not seen by every row
+      const int see_from = edge ? j - t_first - h0 : -1;                     // row h0 + i sees the key from i = see_from on
+      ok = ok && mbar_wait(bar_ready(it), 0, fail);
+      ok = __all_sync(0xffffffffu, ok);
+      tc_fence_after();
+      uint32_t sr[RH];
+      auto subtract_references = [&]() {
+#pragma unroll
+        for (int i = 0; i < RH; i += 4) {
+          const float4 m = *reinterpret_cast<const float4 *>(s_m + h0 + i);
+          sr[i] = __float_as_uint(fmaf(__uint_as_float(sr[i]), sc, -m.x));
+          sr[i + 1] = __float_as_uint(fmaf(__uint_as_float(sr[i + 1]), sc, -m.y));
+          sr[i + 2] = __float_as_uint(fmaf(__uint_as_float(sr[i + 2]), sc, -m.z));
+          sr[i + 3] = __float_as_uint(fmaf(__uint_as_float(sr[i + 3]), sc, -m.w));
+        }
+        if (edge)
+#pragma unroll
+          for (int i = 0; i < RH; ++i)
+            if (i < see_from) sr[i] = 0xff800000u;     // -inf
+      };
+      tmem_load<RH>(t_lane + it * R, sr);
+      bool fresh = it == 0, raise = true;
+      if (fresh && !edge) {                            // a first reference: the largest logit of four of the chunk's keys
+        if (lane == 0)
+#pragma unroll
+          for (int i = 0; i < RH; i += 4)
+            *reinterpret_cast<uint4 *>(s_red + quad * R + h0 + i) = make_uint4(sr[i], sr[i + 1], sr[i + 2], sr[i + 3]);
+        bar_sync(1 + half, 128);
+        if (quad == 0 && lane < RH) {
+          const int r = h0 + lane;
+          s_m[r] = sc * fmaxf(fmaxf(s_red[r], s_red[R + r]), fmaxf(s_red[2 * R + r], s_red[3 * R + r]));
+        }
+        bar_sync(1 + half, 128);
+        fresh = false;
+      }
+      if (!fresh) {
+        subtract_references();
+        float mx = -INFINITY;
+#pragma unroll
+        for (int i = 0; i < RH; ++i) mx = fmaxf(mx, __uint_as_float(sr[i]));
+        raise = bar_any(1 + half, 128, mx > kHeldLazy);
+      }
+      if (raise) {                                     // new references: column maxima over the half's four warps
+        float mine = -INFINITY;
+        tmem_load<RH>(t_lane + it * R, sr);
+#pragma unroll
+        for (int i = 0; i < RH; ++i) {
+          const float mx = warp_max(i >= see_from ? __uint_as_float(sr[i]) * sc : -INFINITY);
+          if (lane == i) mine = mx;
+        }
+        s_red[quad * R + h0 + lane] = mine;
+        bar_sync(1 + half, 128);
+        if (quad == 0) {
+          const int r = h0 + lane;
+          const float mx = fmaxf(fmaxf(s_red[r], s_red[R + r]), fmaxf(s_red[2 * R + r], s_red[3 * R + r]));
+          const float old = fresh ? 0.f : s_m[r];
+          const bool up = mx > -INFINITY && (fresh || mx > old);
+          s_m[r] = up ? mx : old;
+          s_red[r] = up ? fast_exp2(old - mx) : 1.f;
+        }
+        bar_sync(1 + half, 128);
+        if (it > 0)
+#pragma unroll
+          for (int i = 0; i < RH; ++i) l[i] *= s_red[h0 + i];
+        tmem_load<RH>(t_lane + it * R, sr);
+        subtract_references();
+      }
+#pragma unroll
+      for (int i = 0; i < RH; ++i) l[i] += fast_exp2(__uint_as_float(sr[i]));
+    }
+    if (!ok) s_fail = 1;
+    // the rows' sums over the CTA's keys, to every CTA of the cluster
+    const float sum = column_reduce<RH>(l, lane, [](float x, float z) { return x + z; });
+    bar_sync(1 + half, 128);                           // (the factors in s_red have been read)
+    s_red[quad * R + h0 + lane] = sum;
+    bar_sync(3, 256);
+  }
+  __syncwarp();
+  if (n_ctas > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // every peer's barrier is set up
+  if (warp < 8) {
+    // (a row that saw no key here counts for nothing: its reference may be below every other)
+    const int r = tid & (R - 1);
+    const float lr = n_it > 0 ? (s_red[r] + s_red[R + r]) + (s_red[2 * R + r] + s_red[3 * R + r]) : 0.f;
+    const float mr = lr > 0.f ? s_m[r] : -INFINITY;
+    if (tid < R) peer[rank * R + r] = make_float2(mr, lr);
+    for (int to = tid / R; to < n_ctas; to += 256 / R)
+      if (to != rank)
+        st_async_f32x2(map_to_cta(smem_u32(peer + rank * R + r), to), mr, lr, map_to_cta(bar_recv, to));
+    if (n_ctas > 1) {
+      const bool landed = mbar_wait(bar_recv, 0, fail);
+      if (!landed) s_fail = 1;
+    }
+    bar_sync(3, 256);
+    if (tid < R) {
+      float m = -INFINITY, sum = 0.f;
+      for (int k = 0; k < n_ctas; ++k) m = fmaxf(m, peer[k * R + tid].x);
+      for (int k = 0; k < n_ctas; ++k) sum += peer[k * R + tid].y * fast_exp2(peer[k * R + tid].x - m);
+      s_c[tid] = tid < rows && sum > 0.f ? m + log2f(sum) : INFINITY;        // (rows past the last give 0)
+    }
+    bar_sync(3, 256);
+    // ---- pass B: the visual keys' sums over the rows ----
+    const bool good = s_fail == 0;
+    float *out = partial + (((long long)b * n_q_heads + h) * n_row_blocks + qb) * m_max;
+    auto visual = [&](int it) { return (c_begin + it) * kChunk < y.vs + y.nv && (c_begin + it + 1) * kChunk > y.vs; };
+    float mine[kHeld];
+#pragma unroll
+    for (int it = 0; it < kHeld; ++it) {
+      mine[it] = 0.f;
+      if (it < n_it && good && visual(it)) {           // (uniform)
+        uint32_t sr[RH];
+        tmem_load<RH>(t_lane + it * R, sr);
+        float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+        for (int i = 0; i < RH; i += 4) {
+          const float4 c = *reinterpret_cast<const float4 *>(s_c + h0 + i);
+          a0 += fast_exp2(fmaf(__uint_as_float(sr[i]), sc, -c.x));
+          a1 += fast_exp2(fmaf(__uint_as_float(sr[i + 1]), sc, -c.y));
+          a0 += fast_exp2(fmaf(__uint_as_float(sr[i + 2]), sc, -c.z));
+          a1 += fast_exp2(fmaf(__uint_as_float(sr[i + 3]), sc, -c.w));
+        }
+        mine[it] = a0 + a1;
+        if (half == 1) colsum[it * kChunk + kl] = mine[it];
+      }
+    }
+    bar_sync(3, 256);
+    if (half == 0)
+#pragma unroll
+      for (int it = 0; it < kHeld; ++it) {
+        const int m = (c_begin + it) * kChunk + kl - y.vs;
+        if (it < n_it && good && m >= 0 && m < y.nv) out[m] = mine[it] + colsum[it * kChunk + kl];
+      }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (s_fail && tid == 0) flag_status(dev_status, b, TWIG_DEV_INTERNAL);
+  if (warp == 9) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kHeld * R) : "memory");
+}
+
+// ---- longer prompts, 1. probabilities and per-chunk statistics ----
 // grid (n_groups * n_row_blocks, heads, batch); blockIdx.x = row block * n_groups + group.  A CTA walks
 // `chunks_per_cta` consecutive chunks of its item.  Nine warps in two roles that meet only at mbarriers:
-//   warp 8, one thread: brings the key tiles (TMA boxes of the 4-D map over K: 64 columns x 128 rows,
+//   warp 8, one elected lane: brings the key tiles (TMA boxes of the 4-D map over K: 64 columns x 128 rows,
 //     128-byte swizzle, completion counted on the buffer's barrier) into NBUF buffers, a buffer being
 //     refilled as soon as the product that read it has completed, and issues S(t) = Q K(t)^T into one of
 //     two accumulators in tensor memory as soon as the tile is there and the accumulator has been read;
@@ -95,7 +386,8 @@ ttp_mq_probs_kernel(const __nv_bfloat16 *__restrict__ q_text, int n_text_max, co
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_fail;
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // (uniform for the compiler too: see umma8_kk)
   const int grp = blockIdx.x % n_groups, qb = blockIdx.x / n_groups, h = blockIdx.y, b = blockIdx.z;
   grid_dependency_sync();
   const MqLayout y = mq_layout(prefix_len, vis_start, n_vis, b, k_max_len, m_max, n_text_max);
@@ -165,31 +457,32 @@ ttp_mq_probs_kernel(const __nv_bfloat16 *__restrict__ q_text, int n_text_max, co
   volatile int *fail = &s_fail;
 
   if (warp == kMqSoftWarps) {
-    // ================= tiles and products (one thread) =================
-    if (lane == 0) {
-      constexpr uint32_t kIdesc = instr_desc(kMqRows, kChunk, false);
-      bool ok = true;
-      for (int it = 0; it < n_it; ++it) {
-        const int buf = it % NBUF, acc = it & 1;
-        ok = mbar_wait(bar_full(buf), (it / NBUF) & 1, fail);
-        if (ok && it >= 2) ok = mbar_wait(bar_read(acc), ((it - 2) >> 1) & 1, fail);     // S(it - 2) has been read
-        if (!ok) break;
-        tc_fence_after();
+    // ================= tiles and products (one elected lane; the warp stays together) =================
+    const uint32_t leader = elect_one();
+    constexpr uint32_t kIdesc = instr_desc(kMqRows, kChunk, false);
+    bool ok = true;
+    for (int it = 0; it < n_it; ++it) {
+      const int buf = it % NBUF, acc = it & 1;
+      ok = mbar_wait(bar_full(buf), (it / NBUF) & 1, fail);
+      if (ok && it >= 2) ok = mbar_wait(bar_read(acc), ((it - 2) >> 1) & 1, fail);     // S(it - 2) has been read
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t qd = smem_desc(q_s, 16), kd = smem_desc(k_s + buf * K_BYTES, 16);
+      if constexpr (D == 128) {
+        umma8_kk<kMqRows * 128, kChunk * 128>(leader, tmem + acc * kChunk, qd, kd, kIdesc);
+      } else {
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t qa = q_s + (ks >> 2) * kMqRows * 128 + (ks & 3) * 32;
-          const uint32_t ka = k_s + buf * K_BYTES + (ks >> 2) * kChunk * 128 + (ks & 3) * 32;
-          umma(tmem + acc * kChunk, smem_desc(qa, 16), smem_desc(ka, 16), kIdesc, ks > 0);
-        }
-        umma_commit(bar_ready(acc));
-        if (it + NBUF < n_it) {                       // the buffer is refilled once this product has read it
-          ok = mbar_wait(bar_ready(acc), (it >> 1) & 1, fail);
-          if (!ok) break;
-          load_tile(it + NBUF);
-        }
+        for (int ks = 0; ks < D / 16; ++ks)
+          if (leader) umma(tmem + acc * kChunk, qd + 2 * ks, kd + 2 * ks, kIdesc, ks > 0);
       }
-      if (!ok) s_fail = 1;
+      umma_commit_if(leader, bar_ready(acc));
+      if (it + NBUF < n_it) {                         // the buffer is refilled once this product has read it
+        ok = mbar_wait(bar_ready(acc), (it >> 1) & 1, fail);
+        if (!ok) break;
+        if (leader) load_tile(it + NBUF);
+      }
     }
+    if (!ok && lane == 0) s_fail = 1;
   } else {
     // ================= read-back: statistics and exponentials (warps 0-7) =================
     // accumulator row r sits in lane 32 (r / 16) + r % 16 of tensor memory; warps w and w + 4 read rows
@@ -418,7 +711,7 @@ __global__ void ttp_mq_reduce_kernel(const float *__restrict__ partial, int n_bl
   if (y.ok && y.n_text > 0 && m < y.nv) {
     const int nqb = (y.n_text + kMqRows - 1) / kMqRows;
     const int n_terms = n_q_heads * nqb;             // term t = (head t / nqb, row block t % nqb)
-    constexpr int kBatch = 16;                       // loads in flight; the additions keep the index order
+    constexpr int kBatch = 32;                       // loads in flight; the additions keep the index order
     for (int t0 = 0; t0 < n_terms; t0 += kBatch) {
       float v[kBatch];
 #pragma unroll
@@ -519,42 +812,66 @@ extern "C" twig_status ttp_score_multiquery(const void *q_text, int32_t n_text_m
   if (!mq_key_map(&kmap, twig_k, k_stride_batch, k_stride_head, k_stride_pos, k_max_len, n_kv_heads, batch, head_dim))
     return TWIG_ERR_UNSUPPORTED;                      // (no tensor map: there is no other path)
 
-  // Q, two key tiles, the warps' stages; at least 78 KB so that no more than two CTAs share an SM
-  // (each holds half of its tensor memory)
-  constexpr int kBufs = 2;
-  const size_t smem = std::max<size_t>((size_t)(kMqRows + kBufs * kChunk) * head_dim * 2 + kMqSoftWarps * 16 * (64 * 2 + 16), 78 * 1024);
-  static bool attr_set = false;
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(ttp_mq_probs_kernel<128, kBufs>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) != cudaSuccess ||
-        cudaFuncSetAttribute(ttp_mq_probs_kernel<64, kBufs>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) != cudaSuccess)
-      return TWIG_ERR_CUDA;
-    attr_set = true;
-  }
-  // chunks per CTA: walks long enough to pay for a CTA's start (Q, tensor memory, the first tiles' latency),
-  // about 3.5 CTAs per SM in all (measured on 4 x 32 heads x 24 chunks, per call: 2 chunks 61 us, 4: 53, 6: 51,
-  // 8: 52, 12: 50, 24: 56)
-  const long long total_chunks = (long long)items * n_chunks;
-  const int chunks_per_cta = (int)std::min<long long>(12, std::max<long long>(1, (total_chunks + 517) / 518));
-  const int n_groups = (n_chunks + chunks_per_cta - 1) / chunks_per_cta;
-  {
-    PdlLaunch L(dim3(n_groups * n_blocks, n_q_heads, batch), dim3(kMqThreads), smem, st);
+  // One pass while the logits of a prompt fit the tensor memory of a cluster of eight (4096 keys) and all CTAs are
+  // resident at once.  Beyond, the probabilities go through memory: the single pass computes every
+  // exponential twice, and with more than a wave a CTA's chain of waits is no longer hidden (2 prompts of
+  // 28 heads and 4 row blocks: 92 us in one pass, 78 in three kernels; 1 prompt of 32 heads: 17.6 and 22.8).
+  const int ctas = (n_chunks + kHeld - 1) / kHeld;
+  if (n_chunks <= 8 * kHeld && (long long)ctas * n_q_heads * n_blocks * batch <= 2 * 148) {
+    const int smem_held = head_dim == 128 ? held_smem<128>() : held_smem<64>();
+    static bool held_set = false;
+    if (!held_set) {
+      if (cudaFuncSetAttribute(ttp_mq_held_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, held_smem<128>() > 78 * 1024 ? held_smem<128>() : 78 * 1024) != cudaSuccess ||
+          cudaFuncSetAttribute(ttp_mq_held_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, held_smem<64>() > 78 * 1024 ? held_smem<64>() : 78 * 1024) != cudaSuccess)
+        return TWIG_ERR_CUDA;
+      held_set = true;
+    }
+    // (at least 78 KB, so that no more than two CTAs share an SM: each holds half of its tensor memory)
+    ClusterLaunch L(dim3(ctas, n_q_heads * n_blocks, batch), dim3(kHeldThreads), ctas, st, std::max(smem_held, 78 * 1024));
     const cudaError_t err =
-        head_dim == 128
-            ? cudaLaunchKernelEx(&L.cfg, ttp_mq_probs_kernel<128, kBufs>, q, n_text_max, kmap, k_max_len, prefix_len, vis_start,
-                                 n_vis, n_q_heads, group, scale_log2, n_chunks, n_blocks, n_groups, chunks_per_cta, sc, m_max, dev_status)
-            : cudaLaunchKernelEx(&L.cfg, ttp_mq_probs_kernel<64, kBufs>, q, n_text_max, kmap, k_max_len, prefix_len, vis_start,
-                                 n_vis, n_q_heads, group, scale_log2, n_chunks, n_blocks, n_groups, chunks_per_cta, sc, m_max, dev_status);
+        head_dim == 128 ? cudaLaunchKernelEx(&L.cfg, ttp_mq_held_kernel<128>, q, n_text_max, kmap, k_max_len, prefix_len,
+                                             vis_start, n_vis, n_q_heads, group, scale_log2, n_blocks, sc.partial, m_max, dev_status)
+                        : cudaLaunchKernelEx(&L.cfg, ttp_mq_held_kernel<64>, q, n_text_max, kmap, k_max_len, prefix_len,
+                                             vis_start, n_vis, n_q_heads, group, scale_log2, n_blocks, sc.partial, m_max, dev_status);
     if (err != cudaSuccess) return TWIG_ERR_CUDA;
+  } else {
+    // Q, two key tiles, the warps' stages; at least 78 KB so that no more than two CTAs share an SM
+    // (each holds half of its tensor memory)
+    constexpr int kBufs = 2;
+    const size_t smem = std::max<size_t>((size_t)(kMqRows + kBufs * kChunk) * head_dim * 2 + kMqSoftWarps * 16 * (64 * 2 + 16), 78 * 1024);
+    static bool attr_set = false;
+    if (!attr_set) {
+      if (cudaFuncSetAttribute(ttp_mq_probs_kernel<128, kBufs>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) != cudaSuccess ||
+          cudaFuncSetAttribute(ttp_mq_probs_kernel<64, kBufs>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) != cudaSuccess)
+        return TWIG_ERR_CUDA;
+      attr_set = true;
+    }
+    // chunks per CTA: walks long enough to pay for a CTA's start (Q, tensor memory, the first tiles' latency),
+    // about 3.5 CTAs per SM in all (measured on 4 x 32 heads x 24 chunks, per call: 2 chunks 61 us, 4: 53, 6: 51,
+    // 8: 52, 12: 50, 24: 56)
+    const long long total_chunks = (long long)items * n_chunks;
+    const int chunks_per_cta = (int)std::min<long long>(12, std::max<long long>(1, (total_chunks + 517) / 518));
+    const int n_groups = (n_chunks + chunks_per_cta - 1) / chunks_per_cta;
+    {
+      PdlLaunch L(dim3(n_groups * n_blocks, n_q_heads, batch), dim3(kMqThreads), smem, st);
+      const cudaError_t err =
+          head_dim == 128
+              ? cudaLaunchKernelEx(&L.cfg, ttp_mq_probs_kernel<128, kBufs>, q, n_text_max, kmap, k_max_len, prefix_len, vis_start,
+                                   n_vis, n_q_heads, group, scale_log2, n_chunks, n_blocks, n_groups, chunks_per_cta, sc, m_max, dev_status)
+              : cudaLaunchKernelEx(&L.cfg, ttp_mq_probs_kernel<64, kBufs>, q, n_text_max, kmap, k_max_len, prefix_len, vis_start,
+                                   n_vis, n_q_heads, group, scale_log2, n_chunks, n_blocks, n_groups, chunks_per_cta, sc, m_max, dev_status);
+      if (err != cudaSuccess) return TWIG_ERR_CUDA;
+    }
+    {
+      const int vis_chunks = (m_max + kChunk - 1) / kChunk + 1;       // a span of m_max keys touches at most this many chunks
+      PdlLaunch L(dim3((vis_chunks + kSumChunks - 1) / kSumChunks, n_q_heads * n_blocks, batch), dim3(kSumThreads), 0, st);
+      if (cudaLaunchKernelEx(&L.cfg, ttp_mq_colsum_kernel, n_text_max, k_max_len, prefix_len, vis_start, n_vis, n_q_heads,
+                             n_chunks, n_blocks, sc, m_max) != cudaSuccess)
+        return TWIG_ERR_CUDA;
+    }
   }
   {
-    const int vis_chunks = (m_max + kChunk - 1) / kChunk + 1;       // a span of m_max keys touches at most this many chunks
-    PdlLaunch L(dim3((vis_chunks + kSumChunks - 1) / kSumChunks, n_q_heads * n_blocks, batch), dim3(kSumThreads), 0, st);
-    if (cudaLaunchKernelEx(&L.cfg, ttp_mq_colsum_kernel, n_text_max, k_max_len, prefix_len, vis_start, n_vis, n_q_heads,
-                           n_chunks, n_blocks, sc, m_max) != cudaSuccess)
-      return TWIG_ERR_CUDA;
-  }
-  {
-    PdlLaunch L(dim3((m_max + 255) / 256, batch), dim3(256), 0, st);
+    PdlLaunch L(dim3((m_max + 127) / 128, batch), dim3(128), 0, st);
     if (cudaLaunchKernelEx(&L.cfg, ttp_mq_reduce_kernel, (const float *)sc.partial, n_blocks, n_q_heads, n_text_max,
                            prefix_len, vis_start, n_vis, k_max_len, scores, m_max) != cudaSuccess)
       return TWIG_ERR_CUDA;
