@@ -142,12 +142,13 @@ tree_attn_kernel(const AttnParams p) {
   const __nv_bfloat16 *tk = p.tree_k + ((long long)b * p.n_kv_heads + hk) * p.t_max * D;
   const __nv_bfloat16 *tv = p.tree_v + ((long long)b * p.n_kv_heads + hk) * p.t_max * D;
 
-  auto load_tile = [&](int t, int stage) {
-    constexpr int CHUNKS = KT * C::CPR;
+  // rows [r0, r1) of tile t (zeros past the last key)
+  auto load_rows = [&](int t, int stage, int r0, int r1) {
+    constexpr int PASSES = (KT * C::CPR + C::THREADS - 1) / C::THREADS;
 #pragma unroll
-    for (int i = 0; i < (CHUNKS + C::THREADS - 1) / C::THREADS; ++i) {
-      const int cid = i * C::THREADS + tid;
-      if (CHUNKS % C::THREADS != 0 && cid >= CHUNKS) break;
+    for (int i = 0; i < PASSES; ++i) {
+      const int cid = r0 * C::CPR + i * C::THREADS + tid;
+      if (cid >= r1 * C::CPR) break;
       const int r = cid / C::CPR, c = cid % C::CPR;
       const int vj = t * KT + r;
       const __nv_bfloat16 *sk = ck, *sv = cv;
@@ -166,32 +167,37 @@ tree_attn_kernel(const AttnParams p) {
       cp_async_16(v_s + off, sv, valid);
     }
   };
+  auto load_tile = [&](int t, int stage) { load_rows(t, stage, 0, KT); };
 
   // ---- start the copies first: Q tile (zero rows past the last row) and the first key tiles ----
   constexpr int PRE = C::PRE;
-  bool prefetched[PRE > 0 ? PRE : 1];
   if (p.early_prefix) {
 #pragma unroll
     for (int s = 0; s < PRE; ++s) {
       const int t = t_begin + s;
-      prefetched[s] = t < t_end && t * KT + KT <= L;      // wholly inside the cached prefix
-      if (prefetched[s]) load_tile(t, s);
+      if (t < t_end) load_rows(t, s, 0, max(0, min(KT, L - t * KT)));     // what lies inside the cached prefix
       cp_async_commit();
     }
   }
-  auto load_q = [&]() {
-    constexpr int CHUNKS = ROWS * C::CPR;
+  constexpr int Q_PASSES = (ROWS * C::CPR + C::THREADS - 1) / C::THREADS;
+  auto q_source = [&](int i) -> const __nv_bfloat16 * {       // of this thread's i-th chunk (null: zeros)
+    const int cid = i * C::THREADS + tid, gr = row0 + cid / C::CPR;
+    if (gr >= rows_total) return nullptr;
+    const int node = p.group == 1 ? gr : gr / p.group;
+    return p.q + (((long long)b * p.t_max + node) * p.n_q_heads + hk * p.group + (gr - node * p.group)) * D + cid % C::CPR * 8;
+  };
+  // (the small variants have the registers to work the addresses out before the wait)
+  const __nv_bfloat16 *q_src[C::RECV_OWN ? Q_PASSES : 1];
+  if (C::RECV_OWN)
 #pragma unroll
-    for (int i = 0; i < (CHUNKS + C::THREADS - 1) / C::THREADS; ++i) {
+    for (int i = 0; i < Q_PASSES; ++i) q_src[C::RECV_OWN ? i : 0] = q_source(i);
+  auto load_q = [&]() {
+#pragma unroll
+    for (int i = 0; i < Q_PASSES; ++i) {
       const int cid = i * C::THREADS + tid;
-      if (CHUNKS % C::THREADS != 0 && cid >= CHUNKS) break;
-      const int r = cid / C::CPR, c = cid % C::CPR;
-      const int gr = row0 + r;
-      const bool valid = gr < rows_total;
-      const int node = valid ? gr / p.group : 0, g = valid ? gr % p.group : 0;
-      const __nv_bfloat16 *src =
-          p.q + (((long long)b * p.t_max + node) * p.n_q_heads + hk * p.group + g) * D + c * 8;
-      cp_async_16(q_s + tile_off<ROWS>(r, c), src, valid);
+      if ((ROWS * C::CPR) % C::THREADS != 0 && cid >= ROWS * C::CPR) break;
+      const __nv_bfloat16 *src = C::RECV_OWN ? q_src[C::RECV_OWN ? i : 0] : q_source(i);
+      cp_async_16(q_s + tile_off<ROWS>(cid / C::CPR, cid % C::CPR), src ? src : p.q, src != nullptr);
     }
   };
   if (!p.early_prefix) {
@@ -248,7 +254,7 @@ tree_attn_kernel(const AttnParams p) {
     load_q();
 #pragma unroll
     for (int s = 0; s < PRE; ++s)
-      if (t_begin + s < t_end && !prefetched[s]) load_tile(t_begin + s, s);
+      if (t_begin + s < t_end) load_rows(t_begin + s, s, max(0, min(KT, L - (t_begin + s) * KT)), KT);
     cp_async_commit();
     cp_async_wait<0>();
   }
@@ -477,39 +483,53 @@ tree_attn_kernel(const AttnParams p) {
     __syncthreads();                            // all warps are done with the stage ring
   }
   {
-    // The two lanes of a quad pair swap halves so that each holds four consecutive floats of one
-    // row: even lanes of the pair keep the low row, odd lanes the high row; 16-byte stores.
-    const bool odd = tq & 1;
-    const int r = odd ? r_hi : r_lo;
+    // The four lanes of a quad transpose what they hold of two 8-column groups of their two rows, so that each
+    // has one group of one row: lanes 0 and 1 of the low row, 2 and 3 of the high row; 16-byte stores.
+    // (8-byte stores of half as many columns took 0.1 us longer to leave)
+    auto row_factor = [](float m_, float l_, float amax, float &up) {
+      // (a row that saw no key in this split carries m = -inf and counts for nothing)
+      const float inv_l = m_ > -INFINITY && l_ > 0.f ? 1.f / l_ : 0.f;
+      float down;
+      row_scale(amax * inv_l, down, up);
+      return inv_l * down;
+    };
+    float up_lo, up_hi;
+    const float f_lo = row_factor(m_lo, l_lo, amax_lo, up_lo), f_hi = row_factor(m_hi, l_hi, amax_hi, up_hi);
+    const bool high = tq & 2, odd = tq & 1;
+    const int r = high ? r_hi : r_lo;
     const int owner = r / rows_per, lr = r % rows_per;
     const int slot = split * rows_per + lr;
     unsigned char *ro = recv + (size_t)slot * D * 2;
-    const float my_l = odd ? l_hi : l_lo;
-    // (a row that saw no key in this split carries m = -inf and counts for nothing)
-    const bool seen = (odd ? m_hi : m_lo) > -INFINITY && my_l > 0.f;
-    const float inv_l = seen ? 1.f / my_l : 0.f;
-    float down, up;
-    row_scale((odd ? amax_hi : amax_lo) * inv_l, down, up);
     const bool remote = owner != split;           // (n_splits == 1: never)
     const uint32_t ro_c = remote ? map_to_cta(smem_u32(ro), owner) : 0u;
     const uint32_t bar_c = remote ? map_to_cta(recv_bar, owner) : 0u;
 #pragma unroll
-    for (int i = 0; i < OT; ++i) {
-      const float s0 = odd ? o[i][0] : o[i][2], s1 = odd ? o[i][1] : o[i][3];
-      const float g0 = __shfl_xor_sync(0xffffffffu, s0, 1), g1 = __shfl_xor_sync(0xffffffffu, s1, 1);
-      const float4 v = odd ? make_float4(g0, g1, o[i][2], o[i][3]) : make_float4(o[i][0], o[i][1], g0, g1);
-      const uint32_t h0 = pack_f16(v.x * inv_l * down, v.y * inv_l * down), h1 = pack_f16(v.z * inv_l * down, v.w * inv_l * down);
+    for (int i = 0; i < OT; i += 2) {
+      const uint32_t w0 = pack_f16(o[i][0] * f_lo, o[i][1] * f_lo), w1 = pack_f16(o[i + 1][0] * f_lo, o[i + 1][1] * f_lo);
+      const uint32_t w2 = pack_f16(o[i][2] * f_hi, o[i][3] * f_hi), w3 = pack_f16(o[i + 1][2] * f_hi, o[i + 1][3] * f_hi);
+      const uint32_t g0 = __shfl_xor_sync(0xffffffffu, odd ? w0 : w1, 1), g1 = __shfl_xor_sync(0xffffffffu, odd ? w2 : w3, 1);
+      const uint32_t a0 = odd ? g0 : w0, a1 = odd ? w1 : g0;        // low row, group i + odd: columns of the lane pair
+      const uint32_t b0 = odd ? g1 : w2, b1 = odd ? w3 : g1;        // high row
+      const uint32_t h0 = __shfl_xor_sync(0xffffffffu, high ? a0 : b0, 2), h1 = __shfl_xor_sync(0xffffffffu, high ? a1 : b1, 2);
+      const uint4 v = high ? make_uint4(h0, h1, b0, b1) : make_uint4(a0, a1, h0, h1);
       // 8-column groups of a row are XOR-swizzled by the row to spread banks
-      const int off = ((((wn * OT + i) ^ (lr & 7)) << 3) + (tq >> 1) * 4) * 2;
-      if (remote) st_async_b32x2(ro_c + off, h0, h1, bar_c);
-      else *reinterpret_cast<uint2 *>(ro + off) = make_uint2(h0, h1);
+      const int off = ((wn * OT + i + odd) ^ (lr & 7)) << 4;
+      if (remote) st_async_b32x4(ro_c + off, v.x, v.y, v.z, v.w, bar_c);
+      else *reinterpret_cast<uint4 *>(ro + off) = v;
     }
-    if (wn == 0 && tq < 2) {
-      const float mm = seen ? (odd ? m_hi : m_lo) : -INFINITY, ll = seen ? my_l : 0.f;
+    if (wn == 0 && !odd) {
+      const float my_l = high ? l_hi : l_lo, my_m = high ? m_hi : m_lo, up = high ? up_hi : up_lo;
+      const bool seen = my_m > -INFINITY && my_l > 0.f;
+      const float mm = seen ? my_m : -INFINITY, ll = seen ? my_l : 0.f;
       if (remote) st_async_f32x4(map_to_cta(smem_u32(r_ml + slot), owner), mm, ll, up, 0.f, bar_c);
       else r_ml[slot] = make_float4(mm, ll, up, 0.f);
     }
   }
+  // where this thread's first columns go (worked out while the peers' bytes are on their way)
+  constexpr int TPR = D / 4;                          // threads per row, 4 floats each
+  constexpr int RPP = C::THREADS / TPR;               // rows per pass
+  const int c4 = (tid % TPR) * 4;
+  const int gr0 = row0 + split * rows_per + tid / TPR, node0 = p.group == 1 ? gr0 : gr0 / p.group;
   if (n_splits > 1) {
     __syncwarp();                     // the lanes' own-share stores come before lane 0's arrival
     if (lane == 0) mbar_arrive(recv_bar);
@@ -533,40 +553,37 @@ tree_attn_kernel(const AttnParams p) {
 
   if (p.early_query) asm volatile("griddepcontrol.wait;" ::: "memory");     // stores are ordered after the predecessor
   {
-    constexpr int TPR = D / 4;                        // threads per row, 4 floats each
-    constexpr int RPP = C::THREADS / TPR;             // rows per pass
-    const int c4 = (tid % TPR) * 4;
     for (int lr = tid / TPR; lr < rows_per; lr += RPP) {
       const int gr = row0 + split * rows_per + lr;
       if (gr >= rows_total) continue;
-      float mv[8];
+      const int col = (((c4 >> 3) ^ (lr & 7)) << 3) + (c4 & 7);
+      float4 ml[8];
+      uint2 raw[8];
       float mstar = -INFINITY;
 #pragma unroll
       for (int sd = 0; sd < 8; ++sd) {
-        mv[sd] = sd < n_splits ? r_ml[sd * rows_per + lr].x : -INFINITY;
-        mstar = fmaxf(mstar, mv[sd]);
+        const bool there = sd < n_splits;
+        const int at = there ? sd * rows_per + lr : lr;
+        ml[sd] = r_ml[at];
+        raw[sd] = *reinterpret_cast<const uint2 *>(recv + ((size_t)at * D + col) * 2);
+        mstar = fmaxf(mstar, ml[sd].x);               // (a split that is not there repeats the first)
       }
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
       float lsum = 0.f;
-      const int col = (((c4 >> 3) ^ (lr & 7)) << 3) + (c4 & 7);
 #pragma unroll
       for (int sd = 0; sd < 8; ++sd) {
-        if (sd < n_splits) {
-          const float4 ml = r_ml[sd * rows_per + lr];
-          const float wl = fast_exp2(mv[sd] - mstar) * ml.y;
-          lsum += wl;
-          const float wgt = wl * ml.z;
-          const uint2 raw = *reinterpret_cast<const uint2 *>(recv + ((size_t)(sd * rows_per + lr) * D + col) * 2);
-          const float2 v01 = unpack_f16(raw.x), v23 = unpack_f16(raw.y);
-          acc.x = fmaf(wgt, v01.x, acc.x);
-          acc.y = fmaf(wgt, v01.y, acc.y);
-          acc.z = fmaf(wgt, v23.x, acc.z);
-          acc.w = fmaf(wgt, v23.y, acc.w);
-        }
+        if (sd >= n_splits) break;
+        const float wl = fast_exp2(ml[sd].x - mstar) * ml[sd].y;
+        lsum += wl;
+        const float wgt = wl * ml[sd].z;
+        const float2 v01 = unpack_f16(raw[sd].x), v23 = unpack_f16(raw[sd].y);
+        acc.x = fmaf(wgt, v01.x, acc.x);
+        acc.y = fmaf(wgt, v01.y, acc.y);
+        acc.z = fmaf(wgt, v23.x, acc.z);
+        acc.w = fmaf(wgt, v23.y, acc.w);
       }
       const float inv = 1.f / lsum;
-      const int node = gr / p.group, g = gr % p.group;
-      const int h = hk * p.group + g;
+      const int node = lr == tid / TPR ? node0 : gr / p.group, h = hk * p.group + (gr - node * p.group);
       uint2 packed;
       packed.x = pack_bf16(acc.x * inv, acc.y * inv);
       packed.y = pack_bf16(acc.z * inv, acc.w * inv);
