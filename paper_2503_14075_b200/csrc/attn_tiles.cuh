@@ -8,8 +8,9 @@
 namespace twig {
 
 constexpr int kTileKeys = 128;
-constexpr int kTileBytes = kTileKeys * 128 * 2;    // one K (or V) tile: two 64-column panels, 128-byte swizzle
-constexpr int kPanelBytes = kTileKeys * 128;
+constexpr int kPanelBytes = kTileKeys * 128;       // 64 columns of a K (or V) tile, 128-byte swizzle
+template <int D>
+__host__ __device__ constexpr int tile_bytes() { return D / 64 * kPanelBytes; }
 
 // K and V: the cache in boxes of 128, 32 and 8 rows, the tree's rows in boxes of 8
 struct TileMaps {
@@ -35,14 +36,15 @@ struct TileSource {
   int hk, b, layer, slice;      // slice: b * n_kv_heads + hk
 };
 
-// A tile that lies in the cached prefix: two boxes.  Every lane arrives once on `bar` (count 32).
+// A tile that lies in the cached prefix: a box per panel.  Every lane arrives once on `bar` (count 32).
+template <int D>
 __device__ __forceinline__ void load_whole_tile(const TileMaps &maps, const TileSource &s, bool value, uint32_t dst,
                                                 uint32_t bar, int k0, int lane) {
   if (lane == 0) {
     const CUtensorMap *map = value ? &maps.whole.vmap : &maps.whole.kmap;
-    mbar_arrive_expect_tx(bar, kTileBytes);
+    mbar_arrive_expect_tx(bar, tile_bytes<D>());
     tma_load_5d(dst, map, bar, 0, k0, s.hk, s.b, s.layer);
-    tma_load_5d(dst + kPanelBytes, map, bar, 64, k0, s.hk, s.b, s.layer);
+    if (D == 128) tma_load_5d(dst + kPanelBytes, map, bar, 64, k0, s.hk, s.b, s.layer);
   } else {
     mbar_arrive(bar);
   }
@@ -52,6 +54,7 @@ __device__ __forceinline__ void load_whole_tile(const TileMaps &maps, const Tile
 // cp.async cost one warp 1.3 us to issue).  Rows of V between the prefix end and the tree, and after the
 // tree up to the next multiple of 16 (the product's step in keys), must be zero: they are cleared once the
 // boxes have landed on `bar_raw` (count 1).  Every lane arrives once on `bar`; false: the wait ran out.
+template <int D>
 __device__ __forceinline__ bool load_edge_tile(const TileMaps &maps, const TileSource &s, bool value, uint32_t dst,
                                                uint32_t bar, uint32_t bar_raw, uint32_t &raw_phase, int k0, int lane,
                                                volatile int *fail) {
@@ -60,14 +63,15 @@ __device__ __forceinline__ bool load_edge_tile(const TileMaps &maps, const TileS
   const uint32_t on = value ? bar_raw : bar;
   const int e1 = pre >> 5, e2 = e1 + ((pre & 31) >> 3), e3 = e2 + ((n_tree + 7) >> 3);
   if (lane == 0) {
-    const uint32_t bytes = (uint32_t)(pre + ((n_tree + 7) & ~7)) * 256;
+    const uint32_t bytes = (uint32_t)(pre + ((n_tree + 7) & ~7)) * (D * 2);
     if (value) mbar_arrive_expect_tx(on, bytes);
     else mbar_expect_tx(on, bytes);
   }
   __syncwarp();
-  for (int i = lane; i < 2 * e3; i += 32) {        // both panels of each box
-    const int x = (i & 1) * 64, j = i >> 1;
-    const uint32_t to = dst + (i & 1) * kPanelBytes;
+  constexpr int PANELS = D / 64, CPR = D / 8;      // 16-byte chunks per row
+  for (int i = lane; i < PANELS * e3; i += 32) {   // every panel of each box
+    const int x = i % PANELS * 64, j = i / PANELS;
+    const uint32_t to = dst + i % PANELS * kPanelBytes;
     if (j < e2) {
       const int r = j < e1 ? 32 * j : (pre & ~31) + 8 * (j - e1);
       const CacheMaps &m = j < e1 ? maps.box32 : maps.box8;
@@ -82,9 +86,9 @@ __device__ __forceinline__ bool load_edge_tile(const TileMaps &maps, const TileS
     landed = mbar_wait(bar_raw, raw_phase, fail);
     raw_phase ^= 1;
     const int g0 = min(max(s.L - k0, 0), kTileKeys), t0 = pre + n_tree, t1 = min(kTileKeys, (t0 + 15) & ~15);
-    for (int i = lane; i < (pre - g0 + t1 - t0) * 16; i += 32) {
-      const int q = i >> 4, r = q < pre - g0 ? g0 + q : t0 + q - (pre - g0);
-      asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(dst + ((i >> 3) & 1) * kPanelBytes + r * 128 + (i & 7) * 16), "r"(0u) : "memory");
+    for (int i = lane; i < (pre - g0 + t1 - t0) * CPR; i += 32) {
+      const int q = i / CPR, r = q < pre - g0 ? g0 + q : t0 + q - (pre - g0);
+      asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(dst + (i % CPR >> 3) * kPanelBytes + r * 128 + (i & 7) * 16), "r"(0u) : "memory");
     }
     fence_async_smem();
   }

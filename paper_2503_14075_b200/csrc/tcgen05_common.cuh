@@ -67,6 +67,14 @@ __device__ __forceinline__ void umma8_kk(uint32_t leader, uint32_t d, uint64_t a
       TWIG_MMA_SS("t") TWIG_STEP("2", "2") TWIG_MMA_SS("t") TWIG_STEP("2", "2") TWIG_MMA_SS("t") TWIG_STEP("2", "2") TWIG_MMA_SS("t") "}"
       ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(leader), "n"((PA >> 4) - 6), "n"((PB >> 4) - 6) : "memory");
 }
+// one panel (K = 64): four steps
+__device__ __forceinline__ void umma4_kk(uint32_t leader, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
+  asm volatile(
+      "{\n\t.reg .pred p, q, t;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 q, %4, 0;\n\tsetp.ne.b32 t, 1, 0;\n\tsetp.ne.b32 p, 0, 0;\n\t"
+      "mov.b64 a, %1;\n\tmov.b64 b, %2;\n\t"
+      TWIG_MMA_SS("p") TWIG_STEP("2", "2") TWIG_MMA_SS("t") TWIG_STEP("2", "2") TWIG_MMA_SS("t") TWIG_STEP("2", "2") TWIG_MMA_SS("t") "}"
+      ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(leader) : "memory");
+}
 // D (+)= A B, operands that advance by SA / SB bytes a step; `accumulate`: whether the first step adds to D
 template <int SA, int SB>
 __device__ __forceinline__ void umma8_ss(uint32_t leader, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {

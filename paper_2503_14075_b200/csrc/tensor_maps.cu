@@ -7,8 +7,6 @@
 
 namespace twig {
 
-constexpr int kD = 128;          // head_dim
-
 // ---- tensor maps over the whole K and V cache: dims (d, pos, head, batch, layer) ----
 namespace {
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -18,10 +16,10 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 struct MapKey {
   const void *k, *v;
   long long sl, sb, sh, sp;
-  int n_layers, batch, heads, max_len, box_rows;
+  int n_layers, batch, heads, max_len, head_dim, box_rows;
   bool operator==(const MapKey &o) const {
     return k == o.k && v == o.v && sl == o.sl && sb == o.sb && sh == o.sh && sp == o.sp && n_layers == o.n_layers &&
-           batch == o.batch && heads == o.heads && max_len == o.max_len && box_rows == o.box_rows;
+           batch == o.batch && heads == o.heads && max_len == o.max_len && head_dim == o.head_dim && box_rows == o.box_rows;
   }
 };
 struct MapEntry {
@@ -44,7 +42,7 @@ static EncodeTiledFn encode_tiled() {
 }
 
 static bool encode_cache_map(EncodeTiledFn fn, CUtensorMap *out, const void *base, const MapKey &key) {
-  const cuuint64_t dims[5] = {(cuuint64_t)kD, (cuuint64_t)key.max_len, (cuuint64_t)key.heads, (cuuint64_t)key.batch,
+  const cuuint64_t dims[5] = {(cuuint64_t)key.head_dim, (cuuint64_t)key.max_len, (cuuint64_t)key.heads, (cuuint64_t)key.batch,
                               (cuuint64_t)key.n_layers};
   const cuuint64_t strides[4] = {(cuuint64_t)key.sp * 2, (cuuint64_t)key.sh * 2, (cuuint64_t)key.sb * 2,
                                  (cuuint64_t)key.sl * 2};
@@ -70,7 +68,7 @@ bool cache_maps(const AttnParams &p, int box_rows, CacheMaps *out) {
   // strides must be multiples of 16 bytes, and every dimension but the last needs stride * extent in range
   if (p.c_sp <= 0 || p.c_sh <= 0 || p.c_sb < 0 || p.c_sl < 0) return false;
   MapKey key{p.cache_k0, p.cache_v0, p.n_layers > 1 ? p.c_sl : p.c_sp, p.batch > 1 ? p.c_sb : p.c_sp, p.c_sh, p.c_sp,
-             p.n_layers, p.batch, p.n_kv_heads, p.max_len, box_rows};
+             p.n_layers, p.batch, p.n_kv_heads, p.max_len, p.head_dim, box_rows};
   if (p.n_kv_heads == 1) key.sh = key.sp;      // a stride of an extent-1 dimension is never used
   for (auto &e : table)
     if (e.valid && e.key == key) {
@@ -92,8 +90,8 @@ bool cache_maps(const AttnParams &p, int box_rows, CacheMaps *out) {
 bool tree_maps(const AttnParams &p, int box_rows, CacheMaps *out) {
   const EncodeTiledFn fn = encode_tiled();
   if (!fn) return false;
-  const cuuint64_t dims[3] = {(cuuint64_t)kD, (cuuint64_t)p.t_max, (cuuint64_t)p.batch * p.n_kv_heads};
-  const cuuint64_t strides[2] = {(cuuint64_t)kD * 2, (cuuint64_t)kD * 2 * p.t_max};
+  const cuuint64_t dims[3] = {(cuuint64_t)p.head_dim, (cuuint64_t)p.t_max, (cuuint64_t)p.batch * p.n_kv_heads};
+  const cuuint64_t strides[2] = {(cuuint64_t)p.head_dim * 2, (cuuint64_t)p.head_dim * 2 * p.t_max};
   const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1}, estr[3] = {1, 1, 1};
   auto encode = [&](CUtensorMap *map, const __nv_bfloat16 *base) {
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16 *>(base), dims, strides, box, estr,

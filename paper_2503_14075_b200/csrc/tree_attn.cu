@@ -626,10 +626,16 @@ static twig_status launch_attn(const AttnParams &p, int batch, int n_splits, cud
 
 int pick_splits(int items, int max_tiles, int ctas_per_sm, int forced) {
   if (forced > 0) return forced;
-  int s = 1;
-  // double the key splits while all CTAs still fit in one wave
-  while (s < 8 && items * s * 2 <= ctas_per_sm * 148 && s * 2 <= max_tiles) s *= 2;
-  return s;
+  // Clusters of 1, 2, 4 and 8 CTAs that are resident at once (as the occupancy query answers for a B200: a cluster
+  // stays within a GPC, so eight CTAs of a whole SM each fit 15 times, not 18).  One cluster too many is a second
+  // wave: 16 items in clusters of eight, one CTA per SM, took 15.4 us where 15 items took 8.
+  static const int one[4] = {148, 74, 33, 15}, two[4] = {296, 148, 71, 33};
+  const int *fit = ctas_per_sm == 1 ? one : two;
+  int k = 0;
+  // double the key splits while all CTAs still fit in one wave and at most one of them stays without a tile (three
+  // tiles, 4 heads of 420 rows: 14.2 us in two splits, 11.7 in four)
+  while (k < 3 && items <= fit[k + 1] && (2 << k) <= max_tiles + (max_tiles > 2)) ++k;
+  return 1 << k;
 }
 
 // warps that share the 64 keys of a tile in the 16- and 32-row variants
@@ -647,7 +653,7 @@ static twig_status dispatch_attn(AttnParams &p, int batch, int rows, cudaStream_
   p.row_blocks = (rows + rows_per_cta - 1) / rows_per_cta;
   if ((long long)p.n_kv_heads * p.row_blocks > 65535) return TWIG_ERR_UNSUPPORTED;
   const int max_tiles = (p.max_len + p.t_max + 63) / 64;
-  const int n_splits = pick_splits(batch * p.n_kv_heads * p.row_blocks, max_tiles, 2, p.forced_splits);
+  const int n_splits = pick_splits(batch * p.n_kv_heads * p.row_blocks, max_tiles, rows_per_cta == 128 ? 1 : 2, p.forced_splits);
   switch (rows_per_cta) {
     case 16: return launch_attn<C16>(p, batch, n_splits, st);
     case 32: return launch_attn<C32>(p, batch, n_splits, st);
@@ -705,6 +711,7 @@ extern "C" twig_status tree_verify_attention_ex(const void *q, const void *tree_
   p.n_kv_heads = cache->n_kv_heads;
   p.group = n_q_heads / cache->n_kv_heads;
   p.max_len = cache->max_len;
+  p.head_dim = cache->head_dim;
   p.row_blocks = 1;
   p.overlap = (launch_overlap_enabled() && !(flags & TWIG_ATTN_PLAIN_LAUNCH)) ? 1 : 0;
   p.early_prefix = ((flags & TWIG_ATTN_EARLY_PREFIX) && p.overlap) ? 1 : 0;
@@ -726,15 +733,22 @@ extern "C" twig_status tree_verify_attention_ex(const void *q, const void *tree_
     return kernel == TWIG_ATTN_KERNEL_STREAM ? launch_tree_attn_stream(p, cache->batch, rows, st)
                                              : launch_tree_attn_tcgen05(p, cache->batch, rows, st);
   }
-  if (kernel == TWIG_ATTN_KERNEL_AUTO && umma_ok) {
-    // automatic choice.  The mma.sync kernel is for small, latency-bound calls: few (request, kv head)
-    // pairs and few rows; there the host can only go by the cache's capacity (the lengths are on the
-    // device): at 32 rows and 32 pairs the two kernels cross near 800 keys (250 keys 5.8 against 7.6 us,
-    // 4000 keys 19.1 against 15.6), so capacities below 2048 keep it.  With more than 32 rows they cross
-    // at 250 keys; with more than 74 pairs the tcgen05 kernels are never slower.  (The persistent
-    // kernel measured slower on every shape tried, so it only runs when it is named.)
-    const long long pairs = (long long)cache->batch * cache->n_kv_heads;
-    const bool big = pairs > 74 || rows > 64 || cache->max_len >= (rows > 32 ? 256 : 2048);
+  if (kernel == TWIG_ATTN_KERNEL_AUTO && softmax_scale >= 0.f) {
+    // Automatic choice.  The mma.sync kernel is for small, latency-bound calls; the host can only go by the number
+    // of (request, kv head) pairs and the cache's capacity (the lengths are on the device).  Measured on
+    // chains of layers, pairs x keys (us, mma.sync / tcgen05):
+    //   head_dim 128, 10 rows: 64 x 500 7.2 / 7.9, 64 x 1000 9.8 / 9.1; 26 rows: 64 x 250 7.6 / 7.7, 32 x 250 5.3 / 6.9,
+    //     32 x 500 8.3 / 7.7; 60 rows: 64 x 128 9.0 / 9.0, 16 x 500 9.1 / 8.5, 4 x 1000 8.8 / 8.2; more than 74
+    //     pairs: tcgen05 from 64 keys on; 128 rows or less per pair above 64: always; more rows: 16 blocks of
+    //     128 rows x 250 10.6 / 11.3, 64 x 250 14.1 / 13.1
+    //   head_dim 64 (up to 64 rows): 128 x 500 6.2 / 7.5 (12 rows), 9.2 / 8.3 (30 rows), 128 x 1000 10.5 / 9.2;
+    //     64 x 1000 9.3 / 10.0, 64 x 2000 12.8 / 11.9; 256 x 250 7.5 / 6.9, 256 x 2000 58.8 / 43.4; 4 x 4000 7.6 / 7.2
+    // (The persistent kernel measured slower on every shape tried, so it only runs when it is named.)
+    const long long pairs = (long long)cache->batch * cache->n_kv_heads, keys = pairs * cache->max_len;
+    bool big;
+    if (cache->head_dim == 64) big = rows <= 64 && (keys >= (pairs > 148 ? 60000 : 100000) || cache->max_len >= 4000);
+    else if (rows > 64) big = rows <= 128 || pairs * ((rows + 127) / 128) > 32 || cache->max_len > 256;
+    else big = pairs > 74 || cache->max_len >= 3000 || keys >= (rows > 32 ? 8000 : rows > 16 ? 16000 : 40000);
     if (big) {
       const twig_status us = launch_tree_attn_tcgen05(p, cache->batch, rows, st);
       if (us != TWIG_ERR_UNSUPPORTED) return us;     // no tensor map for this layout: the mma.sync kernel

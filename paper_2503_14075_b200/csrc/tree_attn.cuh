@@ -16,7 +16,7 @@ struct AttnParams {
   __nv_bfloat16 *out;
   float *lse;
   int *dev_status;
-  int t_max, n_q_heads, n_kv_heads, group, max_len, row_blocks;
+  int t_max, n_q_heads, n_kv_heads, group, max_len, row_blocks, head_dim;
   // whole cache (all layers), for the tensor maps of the tcgen05 path
   const __nv_bfloat16 *cache_k0, *cache_v0;
   long long c_sl;
@@ -150,9 +150,9 @@ bool cache_maps(const AttnParams &p, int box_rows, CacheMaps *out);
 // The same over the call's tree rows, dims (d, node, request x head); encoded on every call.
 bool tree_maps(const AttnParams &p, int box_rows, CacheMaps *out);
 
-// tcgen05 path (tree_attn_wide.cu): head_dim 128, rows = t_max * group.
+// tcgen05 path (tree_attn_wide.cu): head_dim 128 (up to 64 rows: 64 too), rows = t_max * group.
 twig_status launch_tree_attn_tcgen05(AttnParams &p, int batch, int rows, cudaStream_t st);
-// the same for rows <= 64, products transposed (tree_attn_narrow.cu)
+// rows <= 64, head_dim 128 or 64, products transposed (tree_attn_narrow.cu)
 twig_status launch_tree_attn_narrow(AttnParams &p, int batch, int rows, cudaStream_t st);
 // persistent tcgen05 path (tree_attn_stream.cu): the same shapes, needs the caller's scratch
 twig_status launch_tree_attn_stream(AttnParams &p, int batch, int rows, cudaStream_t st);

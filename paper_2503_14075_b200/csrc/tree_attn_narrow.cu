@@ -35,17 +35,17 @@ namespace twig {
 
 namespace {
 
-constexpr int kD = 128;                            // head_dim
 constexpr int kKeys = kTileKeys;                  // keys per tile
 constexpr int kThreads = 320;
 constexpr int kSoftWarps = 8;
 constexpr float kLazyMax = 8.f;                    // raise a row's reference only beyond this (log2 units)
 
-template <int R, int SLOTS_, int MIN_CTAS>
+template <int D, int R, int SLOTS_, int MIN_CTAS>
 struct NarrowCfg {
   static constexpr int SLOTS = SLOTS_;
+  static constexpr int TILE_BYTES = tile_bytes<D>();
   static constexpr int RH = R / 2;                 // rows per softmax thread
-  static constexpr int Q_BYTES = R * kD * 2;       // two 64-column panels of R x 128 B
+  static constexpr int Q_BYTES = R * D * 2;        // 64-column panels of R x 128 B
   static constexpr int P_ROW = R * 2;              // bytes of a key's probabilities
   // A product of eight instructions takes 800 cycles from its issue to the barrier that reports it, as
   // long as the softmax of a tile: with one P buffer the two alternate.  Two CTAs on an SM fill each
@@ -55,14 +55,14 @@ struct NarrowCfg {
   static constexpr int P_BYTES = P_BUFS * P_ONE;
   // units requested before the predecessor is waited for; the rest of the ring queues up behind Q, not in
   // front of it (Q took 3.4 us behind 192 KB per SM)
-  static constexpr int PRE_UNITS = 2;
-  static constexpr int RING_BYTES = SLOTS * kTileBytes;
+  static constexpr int PRE_UNITS = 256 / D;
+  static constexpr int RING_BYTES = SLOTS * TILE_BYTES;
   static constexpr int SMEM_BYTES = Q_BYTES + P_BYTES + RING_BYTES;
   static constexpr uint32_t TMEM_COLS = R == 64 ? 256 : R == 32 ? 128 : 64;     // S^T twice, O^T: 3 R columns
   static constexpr uint32_t O_COL = 2 * R;
   // P^T is MN-major with rows of P_ROW bytes: the swizzle of that width
   static constexpr int P_LAYOUT = R == 64 ? 2 : R == 32 ? 4 : 6;
-  static_assert(2 * R * kD * 4 <= RING_BYTES, "the split merge stages and receives fp32 rows in the ring");
+  static_assert(PRE_UNITS <= SLOTS && 2 * R * D * 4 <= RING_BYTES, "the split merge stages and receives fp32 rows in the ring");
 };
 
 // shared-memory matrix descriptor with a choice of swizzle (2: 128 B, 4: 64 B, 6: 32 B)
@@ -77,12 +77,12 @@ __device__ __forceinline__ void bulk_to_cluster(uint32_t dst, uint32_t src, uint
                "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-template <int R, int SLOTS, int MIN_CTAS>
+template <int D, int R, int SLOTS, int MIN_CTAS>
 __global__ void __launch_bounds__(kThreads, MIN_CTAS)
 tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps maps) {
-  using C = NarrowCfg<R, SLOTS, MIN_CTAS>;
+  using C = NarrowCfg<D, R, SLOTS, MIN_CTAS>;
   using RowBits = typename std::conditional<R == 64, unsigned long long, unsigned int>::type;
-  constexpr int RH = C::RH;
+  constexpr int RH = C::RH, CPR = D / 8;           // 16-byte chunks of a row
   extern __shared__ __align__(1024) unsigned char smem[];
   // (static shared memory stays below 1 KB: two CTAs of the largest ring fill an SM exactly)
   __shared__ RowBits s_vis[TWIG_MAX_NODES];        // bit r of entry j: row r of this CTA sees tree node j
@@ -127,7 +127,7 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
     mbar_init(bar_recv, 1);
     mbar_init(bar_raw, 1);
     if (n_splits > 1)                              // every peer's O rows and (m, l)
-      mbar_arrive_expect_tx(bar_recv, (uint32_t)((n_splits - 1) * rows_per * (kD * 4 + 16)));
+      mbar_arrive_expect_tx(bar_recv, (uint32_t)((n_splits - 1) * rows_per * (D * 4 + 16)));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 9) {
@@ -187,7 +187,7 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
   const TileSource source{L, L8, NK, hk, b, p.layer, b * p.n_kv_heads + hk};
   auto load_whole = [&](int u) {
     const int slot = u % SLOTS;
-    load_whole_tile(maps, source, unit_is_v(u), ring_s + slot * kTileBytes, bar_full(slot), unit_tile(u) * kKeys, lane);
+    load_whole_tile<D>(maps, source, unit_is_v(u), ring_s + slot * C::TILE_BYTES, bar_full(slot), unit_tile(u) * kKeys, lane);
   };
   const int n_first = min(n_units, C::PRE_UNITS);
   if (warp == 8)
@@ -222,7 +222,7 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
       if (unit_in_prefix(u)) {
         load_whole(u);
       } else {
-        ok = load_edge_tile(maps, source, unit_is_v(u), ring_s + u % SLOTS * kTileBytes, bar_full(u % SLOTS), bar_raw, raw_phase,
+        ok = load_edge_tile<D>(maps, source, unit_is_v(u), ring_s + u % SLOTS * C::TILE_BYTES, bar_full(u % SLOTS), bar_raw, raw_phase,
                             unit_tile(u) * kKeys, lane, fail);
         ok = __all_sync(0xffffffffu, ok);
       }
@@ -233,7 +233,7 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
     {
       const uint32_t leader = elect_one();
       // S^T: A = K (K-major), B = Q (K-major); O^T: A = V (MN-major), B = P^T (MN-major)
-      constexpr uint32_t kIdescS = instr_desc(128, R, false), kIdescO = instr_desc(128, R, true) | (1u << 15);
+      constexpr uint32_t kIdescS = instr_desc(128, R, false), kIdescO = instr_desc(D, R, true) | (1u << 15);
       bool ok = true;
       auto wait_full = [&](int u) {
         if (ok) ok = mbar_wait(bar_full(u % SLOTS), (u / SLOTS) & 1, fail);
@@ -242,8 +242,9 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
         const int u = it == 0 ? 0 : 2 * it - 1;
         wait_full(u);
         if (!ok) return;
-        umma8_kk<kPanelBytes, R * 128>(leader, tmem + (it & 1) * R, smem_desc(ring_s + (u % SLOTS) * kTileBytes, 16),
-                                       smem_desc(q_s, 16), kIdescS);
+        const uint64_t kd = smem_desc(ring_s + (u % SLOTS) * C::TILE_BYTES, 16), qd = smem_desc(q_s, 16);
+        if constexpr (D == 128) umma8_kk<kPanelBytes, R * 128>(leader, tmem + (it & 1) * R, kd, qd, kIdescS);
+        else umma4_kk(leader, tmem + (it & 1) * R, kd, qd, kIdescS);
         umma_commit_if(leader, bar_s(it & 1));
         umma_commit_if(leader, bar_empty(u % SLOTS));
       };
@@ -258,7 +259,7 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
         wait_full(u);
         if (!ok) break;
         tc_fence_after();
-        const uint64_t vd = smem_desc(ring_s + (u % SLOTS) * kTileBytes, kPanelBytes);
+        const uint64_t vd = smem_desc(ring_s + (u % SLOTS) * C::TILE_BYTES, kPanelBytes);
         const uint64_t pd = smem_desc_of(p_s + it % C::P_BUFS * C::P_ONE, 16, 8 * C::P_ROW, C::P_LAYOUT);
         const int steps = (min(kKeys, NK - (t_begin + it) * kKeys) + 15) >> 4;     // 16 keys each
         if (steps == kKeys / 16) umma8_ss<2048, 16 * C::P_ROW>(leader, tmem + C::O_COL, vd, pd, kIdescO, it > 0);
@@ -278,11 +279,12 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
     bool ok = true;
     if (n_my > 0) {                                // Q (zero rows past the request's last row)
 #pragma unroll
-      for (int i = 0; i < R / 16; ++i) {
-        const int r = i * 16 + (tid >> 4), c = tid & 15;
+      for (int i = 0; i < (R * CPR + 255) / 256; ++i) {
+        const int r = i * (256 / CPR) + tid / CPR, c = tid % CPR;
+        if (R * CPR < 256 && r >= R) break;
         const bool valid = row0 + r < rows_total;
         const int gr = valid ? row0 + r : 0, node = gr / p.group, g = gr - node * p.group;
-        const __nv_bfloat16 *src = p.q + (((long long)b * p.t_max + node) * p.n_q_heads + hk * p.group + g) * kD + c * 8;
+        const __nv_bfloat16 *src = p.q + (((long long)b * p.t_max + node) * p.n_q_heads + hk * p.group + g) * D + c * 8;
         cp_async_16(q_s + (c >> 3) * R * 128 + r * 128 + (((c & 7) ^ (r & 7)) << 4), src, valid);
       }
       cp_async_commit();
@@ -439,12 +441,13 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
   __syncwarp();
   // every unit that was requested has been used, every product has completed: the ring is free
   if (n_splits > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  float *stage = reinterpret_cast<float *>(smem + C::Q_BYTES + C::P_BYTES);     // [row][128] fp32
+  float *stage = reinterpret_cast<float *>(smem + C::Q_BYTES + C::P_BYTES);     // [row][D] fp32
   if (warp < kSoftWarps) {
     uint32_t o[RH];
     if (n_my > 0) tmem_load<RH>(t_lane + C::O_COL + h0, o);
 #pragma unroll
-    for (int i = 0; i < RH; ++i) stage[(h0 + i) * kD + quad * 32 + lane] = n_my > 0 ? __uint_as_float(o[i]) : 0.f;
+    for (int i = 0; i < RH; ++i)                   // (64 rows of O^T: 16 in each quadrant's first lanes)
+      if (D == 128 || lane < 16) stage[(h0 + i) * D + quad * (D / 4) + lane] = n_my > 0 ? __uint_as_float(o[i]) : 0.f;
     if (n_splits > 1) fence_async_smem();          // (the rows leave by bulk copies)
   }
   tc_fence_before();
@@ -454,7 +457,7 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
   const bool ok = s_fail == 0;
   if (!ok && tid == 0) flag_status(p.dev_status, b, TWIG_DEV_INTERNAL);
   auto row_sum = [&](int r) { return n_my > 0 ? (s_red[r] + s_red[R + r]) + (s_red[2 * R + r] + s_red[3 * R + r]) : 0.f; };
-  // eight columns of one row (a row is 16 consecutive threads), and its log-sum-exp
+  // eight columns of one row (a row is D / 8 consecutive threads), and its log-sum-exp
   auto store_row8 = [&](int r, int c, const float (&acc)[8], float lsum, float m) {
     const int gr = row0 + r, node = p.group == 1 ? gr : gr / p.group, h = hk * p.group + (gr - node * p.group);
     const float inv = 1.f / lsum;
@@ -463,7 +466,7 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
     packed.y = pack_bf16(acc[2] * inv, acc[3] * inv);
     packed.z = pack_bf16(acc[4] * inv, acc[5] * inv);
     packed.w = pack_bf16(acc[6] * inv, acc[7] * inv);
-    st_16(p.out + (((long long)b * p.t_max + node) * p.n_q_heads + h) * kD + c, packed);
+    st_16(p.out + (((long long)b * p.t_max + node) * p.n_q_heads + h) * D + c, packed);
     if (p.lse && c == 0)
       p.lse[((long long)b * p.n_q_heads + h) * p.t_max + node] = (m + log2f(lsum)) * 0.6931471805599453f;
   };
@@ -471,12 +474,12 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
   if (n_splits == 1) {
     if (ok) {
 #pragma unroll
-      for (int k = 0; k < (R * 16 + kThreads - 1) / kThreads; ++k) {
-        const int i = tid + k * kThreads, r = i >> 4, c = (i & 15) * 8;
+      for (int k = 0; k < (R * CPR + kThreads - 1) / kThreads; ++k) {
+        const int i = tid + k * kThreads, r = i / CPR, c = i % CPR * 8;
         if (r < n_rows) {
           float acc[8];
-          *reinterpret_cast<float4 *>(acc) = *reinterpret_cast<const float4 *>(stage + r * kD + c);
-          *reinterpret_cast<float4 *>(acc + 4) = *reinterpret_cast<const float4 *>(stage + r * kD + c + 4);
+          *reinterpret_cast<float4 *>(acc) = *reinterpret_cast<const float4 *>(stage + r * D + c);
+          *reinterpret_cast<float4 *>(acc + 4) = *reinterpret_cast<const float4 *>(stage + r * D + c + 4);
           store_row8(r, c, acc, row_sum(r), s_m[r]);
         }
       }
@@ -485,13 +488,13 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
   }
 
   // ---- merge the key splits of the cluster: every CTA owns R / n_splits rows ----
-  // received O rows: [sender][owned row][128] fp32 behind the stage; (m, l): [sender][owned row] in P's place
-  float *recv = stage + R * kD;
+  // received O rows: [sender][owned row][D] fp32 behind the stage; (m, l): [sender][owned row] in P's place
+  float *recv = stage + R * D;
   float4 *recv_ml = reinterpret_cast<float4 *>(smem + C::Q_BYTES);
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // every peer has left its key loop
   if (warp == 0 && lane < n_splits && lane != split) {                    // one copy per owner
-    const uint32_t dst = map_to_cta(smem_u32(recv + (size_t)split * rows_per * kD), lane);
-    bulk_to_cluster(dst, smem_u32(stage + (size_t)lane * rows_per * kD), (uint32_t)(rows_per * kD * 4), map_to_cta(bar_recv, lane));
+    const uint32_t dst = map_to_cta(smem_u32(recv + (size_t)split * rows_per * D), lane);
+    bulk_to_cluster(dst, smem_u32(stage + (size_t)lane * rows_per * D), (uint32_t)(rows_per * D * 4), map_to_cta(bar_recv, lane));
   }
   if (tid >= 32 && tid < 32 + R) {
     const int r = tid - 32, owner = r / rows_per;
@@ -504,8 +507,8 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
   const bool landed = mbar_wait(bar_recv, 0, fail);
   if (!landed && tid == 0) flag_status(p.dev_status, b, TWIG_DEV_INTERNAL);
   if (landed && ok)
-    for (int i = tid; i < rows_per * 16; i += kThreads) {
-      const int lr = i >> 4, c = (i & 15) * 8;
+    for (int i = tid; i < rows_per * CPR; i += kThreads) {
+      const int lr = i / CPR, c = i % CPR * 8;
       if (split * rows_per + lr >= n_rows) break;
       float m = -INFINITY;
       for (int s = 0; s < n_splits; ++s) m = fmaxf(m, recv_ml[s * rows_per + lr].x);
@@ -514,7 +517,7 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
       for (int s = 0; s < n_splits; ++s) {
         const float4 ml = recv_ml[s * rows_per + lr];
         const float w = fast_exp2(ml.x - m);
-        const float *src = (s == split ? stage + (size_t)(split * rows_per + lr) * kD : recv + (size_t)(s * rows_per + lr) * kD) + c;
+        const float *src = (s == split ? stage + (size_t)(split * rows_per + lr) * D : recv + (size_t)(s * rows_per + lr) * D) + c;
         float v[8];
         *reinterpret_cast<float4 *>(v) = *reinterpret_cast<const float4 *>(src);
         *reinterpret_cast<float4 *>(v + 4) = *reinterpret_cast<const float4 *>(src + 4);
@@ -529,12 +532,12 @@ tree_attn_narrow_kernel(const AttnParams p, const __grid_constant__ TileMaps map
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-template <int R, int SLOTS, int MIN_CTAS>
+template <int D, int R, int SLOTS, int MIN_CTAS>
 twig_status launch_narrow(const AttnParams &p, const TileMaps &maps, int batch, int n_splits, cudaStream_t st) {
-  using C = NarrowCfg<R, SLOTS, MIN_CTAS>;
+  using C = NarrowCfg<D, R, SLOTS, MIN_CTAS>;
   static bool attr_set = false;
   if (!attr_set) {
-    if (cudaFuncSetAttribute(tree_attn_narrow_kernel<R, SLOTS, MIN_CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(tree_attn_narrow_kernel<D, R, SLOTS, MIN_CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              C::SMEM_BYTES) != cudaSuccess)
       return TWIG_ERR_CUDA;
     attr_set = true;
@@ -553,7 +556,7 @@ twig_status launch_narrow(const AttnParams &p, const TileMaps &maps, int batch, 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = p.overlap ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, tree_attn_narrow_kernel<R, SLOTS, MIN_CTAS>, p, maps) == cudaSuccess ? TWIG_OK : TWIG_ERR_CUDA;
+  return cudaLaunchKernelEx(&cfg, tree_attn_narrow_kernel<D, R, SLOTS, MIN_CTAS>, p, maps) == cudaSuccess ? TWIG_OK : TWIG_ERR_CUDA;
 }
 
 }  // namespace
@@ -571,11 +574,22 @@ twig_status launch_tree_attn_narrow(AttnParams &p, int batch, int rows, cudaStre
   //   more: two CTAs per SM, whose start and end overlap (T = 64, B = 8, L = 1500: 42.2 against 48.0; T = 32,
   //     B = 16, L = 1500: 67.4 against 80.9).
   const int items = batch * p.n_kv_heads, max_tiles = (p.max_len + p.t_max + kKeys - 1) / kKeys;
-  const bool single = items <= 148 && (rows > 32 || items > 74);
-  const int n_splits = pick_splits(items, max_tiles, single ? 1 : 2, p.forced_splits);
-  if (rows <= 16) return single ? launch_narrow<16, 5, 1>(p, maps, batch, n_splits, st) : launch_narrow<16, 3, 2>(p, maps, batch, n_splits, st);
-  if (rows <= 32) return single ? launch_narrow<32, 5, 1>(p, maps, batch, n_splits, st) : launch_narrow<32, 3, 2>(p, maps, batch, n_splits, st);
-  return single ? launch_narrow<64, 4, 1>(p, maps, batch, n_splits, st) : launch_narrow<64, 2, 2>(p, maps, batch, n_splits, st);
+  // Long caches are an exception where one CTA per SM leaves SMs idle (at most 74 CTAs with all the splits that are
+  // resident at once), and with head_dim 64 always: half the bytes per tile, so the chain of a tile is what
+  // more CTAs hide (T = 60, L = 8000, head_dim 128, 16 items: 26.1 and 22.7, 36 items: 46.0 and 37.5; head_dim 64, 64
+  // items: 43.1 and 32.9; the other way round below 3000 keys, 16 items at 1000 keys: 10.0 and 11.0).
+  const int splits1 = pick_splits(items, max_tiles, 1, p.forced_splits);
+  const bool spread = p.max_len >= 3000 && (p.head_dim == 64 || items * splits1 <= 74);
+  const bool single = items <= 148 && (rows > 32 || items > 74) && !spread;
+  const int n_splits = single ? splits1 : pick_splits(items, max_tiles, 2, p.forced_splits);
+  if (p.head_dim == 64) {
+    if (rows <= 16) return single ? launch_narrow<64, 16, 10, 1>(p, maps, batch, n_splits, st) : launch_narrow<64, 16, 6, 2>(p, maps, batch, n_splits, st);
+    if (rows <= 32) return single ? launch_narrow<64, 32, 10, 1>(p, maps, batch, n_splits, st) : launch_narrow<64, 32, 6, 2>(p, maps, batch, n_splits, st);
+    return single ? launch_narrow<64, 64, 8, 1>(p, maps, batch, n_splits, st) : launch_narrow<64, 64, 5, 2>(p, maps, batch, n_splits, st);
+  }
+  if (rows <= 16) return single ? launch_narrow<128, 16, 5, 1>(p, maps, batch, n_splits, st) : launch_narrow<128, 16, 3, 2>(p, maps, batch, n_splits, st);
+  if (rows <= 32) return single ? launch_narrow<128, 32, 5, 1>(p, maps, batch, n_splits, st) : launch_narrow<128, 32, 3, 2>(p, maps, batch, n_splits, st);
+  return single ? launch_narrow<128, 64, 4, 1>(p, maps, batch, n_splits, st) : launch_narrow<128, 64, 2, 2>(p, maps, batch, n_splits, st);
 }
 
 }  // namespace twig

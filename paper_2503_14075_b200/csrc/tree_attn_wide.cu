@@ -27,6 +27,7 @@ namespace twig {
 namespace {
 
 constexpr int kD = 128;                            // head_dim
+constexpr int kTileBytes = tile_bytes<kD>();
 constexpr int kKeys = kTileKeys;
 constexpr int kRows = 256;                         // rows of a CTA: two streams of 128
 constexpr int kThreads = 384;                      // three warpgroups: registers are shared out between whole ones
@@ -146,7 +147,7 @@ tree_attn_wide_kernel(const AttnParams p, const __grid_constant__ TileMaps maps)
   auto v_unit = [&](int t) { return two ? 2 * t + 1 : t == n_my - 1 ? n_units - 1 : 2 * t + 2; };
   const TileSource source{L, L8, NK, hk, b, p.layer, b * p.n_kv_heads + hk};
   auto load_whole = [&](int u) {
-    load_whole_tile(maps, source, unit_is_v(u), ring_s + u % kSlots * kTileBytes, bar_full(u % kSlots), unit_key(u), lane);
+    load_whole_tile<kD>(maps, source, unit_is_v(u), ring_s + u % kSlots * kTileBytes, bar_full(u % kSlots), unit_key(u), lane);
   };
   const int n_first = min(n_units, kPreUnits);
   if (warp == 8)
@@ -193,7 +194,7 @@ tree_attn_wide_kernel(const AttnParams p, const __grid_constant__ TileMaps maps)
       if (whole) {
         load_whole(u);
       } else {
-        ok = load_edge_tile(maps, source, unit_is_v(u), ring_s + u % kSlots * kTileBytes, bar_full(u % kSlots), bar_raw,
+        ok = load_edge_tile<kD>(maps, source, unit_is_v(u), ring_s + u % kSlots * kTileBytes, bar_full(u % kSlots), bar_raw,
                             raw_phase, unit_key(u), lane, fail);
         ok = __all_sync(0xffffffffu, ok);
       }

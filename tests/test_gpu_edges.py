@@ -46,6 +46,29 @@ def test_tcgen05_attention_tile_edges(tw, nodes, group, kv_len, splits):
     assert np.array_equal(got, early) and np.array_equal(lse, early_lse)
 
 
+@pytest.mark.parametrize("nodes,group,kv_len", ATTN[:6], ids=[f"rows{max(n) * g}" for n, g, L in ATTN[:6]])
+def test_automatic_kernel_choice_head_dim_64(tw, nodes, group, kv_len):
+    """A cache of 4096 keys takes the automatic choice to the tcgen05 kernel's head_dim 64 variants (more (request,
+    head) pairs than SMs, and few), one of 400 to the mma.sync kernel."""
+    d = 64
+    for Hkv, capacity in ((2, 4096), (50, 4096), (2, 400)):
+        keep = min(len(nodes), 2 if Hkv > 2 else 3)
+        nn, L = nodes[:keep] + [0] * (3 - keep), [min(x, capacity - 1) for x in kv_len]
+        wl = _wl(3, Hkv * group, Hkv, d, nn, [4 if x else 0 for x in nn])
+        rng = synth.rng_for(9, 911 + max(nodes) * group)
+        ver = synth.make_verify_inputs(wl, rng, n_layers=1, gain=d ** 0.5)
+        ck, cv = (np.full((1, 3, Hkv, capacity, d), CANARY, dtype=np.uint16) for _ in range(2))
+        k, v = synth.make_cache(wl, rng, max(L) + 1, n_layers=1, gain=d ** 0.5)
+        for b in range(3):
+            ck[0, b, :, :L[b]], cv[0, b, :, :L[b]] = k[0, b, :, :L[b]], v[0, b, :, :L[b]]
+        got, lse, status = run_attention(tw, wl, ver, ck, cv, L)
+        early, early_lse, _ = run_attention(tw, wl, ver, ck, cv, L, early=True)
+        assert not status.any()
+        want, want_lse = oracle_attention(ver, ck[:, :, :, :max(L) + 1], cv[:, :, :, :max(L) + 1], np.array(L))
+        check(got, lse, want, want_lse, ver["n_nodes"])
+        assert np.array_equal(got, early) and np.array_equal(lse, early_lse)
+
+
 # vocabularies around the sizes at which a row is split over 2, 4 and 8 CTAs (bf16: 4096 tokens each, fp32: half)
 VOCABS = [1, 8, 2047, 4096, 4103, 8191, 16385, 32769, 130001]
 
