@@ -266,11 +266,13 @@ tree_attn_wide_kernel(const AttnParams p, const __grid_constant__ TileMaps maps)
     const bool loads_q = two || stream == 0;
     if (n_my > 0 && loads_q) {                     // Q of this stream (zero rows past the request's last row)
       const int first_row = row0 + (two ? stream * 128 : 0), t128 = tid & 127;
+      // (rows stay far below 2^20, so the quotient by multiplication is exact)
+      const float inv_group = 1.f / (float)p.group;
 #pragma unroll 4
       for (int i = 0; i < 16; ++i) {
         const int r = i * 8 + (t128 >> 4), c = t128 & 15;
         const bool valid = first_row + r < rows_total;
-        const int row = valid ? first_row + r : 0, node = row / p.group, g = row - node * p.group;
+        const int row = valid ? first_row + r : 0, node = (int)(((float)row + 0.5f) * inv_group), g = row - node * p.group;
         const __nv_bfloat16 *src = p.q + (((long long)b * p.t_max + node) * p.n_q_heads + hk * p.group + g) * kD + c * 8;
         cp_async_16(q_s + (two ? stream * kQBytes : 0) + (c >> 3) * kPanelBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4), src, valid);
       }
@@ -462,7 +464,19 @@ tree_attn_wide_kernel(const AttnParams p, const __grid_constant__ TileMaps maps)
   unsigned char *recv = smem + 2 * kQBytes;                   // [sender * rows_per + owned row][128] fp16, in the ring
   float4 *r_ml = reinterpret_cast<float4 *>(smem);            // (m, l, row scale, -), in Q's place
   if (tid == 0) mbar_arrive_expect_tx(bar_recv, (uint32_t)((n_splits - 1) * rows_per * (kD * 2 + 16)));
-  cluster.sync();                                             // every CTA has left its key loop
+  // this CTA has left its key loop; the rows' scales are found while the others leave theirs
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  float amax = 0.f;
+  if (have_o) {
+#pragma unroll 1
+    for (int ch = 0; ch < 4; ++ch) {
+      float v[32];
+      load_o(ch, v);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) amax = fmaxf(amax, fabsf(v[i]));
+    }
+  }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (warp < 8) {
     const int rl = row_active ? row_local : 0;
     const int owner = rl / rows_per, lr = rl % rows_per, slot = split * rows_per + lr;
@@ -472,16 +486,6 @@ tree_attn_wide_kernel(const AttnParams p, const __grid_constant__ TileMaps maps)
     // (a row that saw no key in this split carries m = -inf and counts for nothing)
     const bool seen = have_o && row_valid && m_run > -INFINITY && l_run > 0.f;
     const float inv_l = seen ? 1.f / l_run : 0.f;
-    float amax = 0.f;
-    if (have_o) {
-#pragma unroll 1
-      for (int ch = 0; ch < 4; ++ch) {
-        float v[32];
-        load_o(ch, v);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) amax = fmaxf(amax, fabsf(v[i]));
-      }
-    }
     float down, up;
     row_scale(seen ? amax * inv_l : 0.f, down, up);
 #pragma unroll 1
@@ -569,7 +573,10 @@ twig_status launch_tree_attn_tcgen05(AttnParams &p, int batch, int rows, cudaStr
     attr_set = true;
   }
   const int max_tiles = (p.max_len + p.t_max + kKeys - 1) / kKeys;
-  const int n_splits = pick_splits(batch * p.n_kv_heads * p.row_blocks, max_tiles, 1, p.forced_splits);
+  int n_splits = pick_splits(batch * p.n_kv_heads * p.row_blocks, max_tiles, 1, p.forced_splits);
+  // A merge costs 3 us, a tile 1.6 us with different rows in the streams and 0.85 with alternate tiles: halving a
+  // short item does not pay (240 rows, 64 pairs, 3 tiles: 14.1 us whole, 15.6 halved; 72 rows, 9 tiles: 13.8, 14.0).
+  if (p.forced_splits == 0 && (rows > 128 ? n_splits == 2 && max_tiles < 4 : max_tiles < (n_splits == 2 ? 8 : 4))) n_splits = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_splits, p.n_kv_heads * p.row_blocks, batch);
   cfg.blockDim = dim3(kThreads);
