@@ -11,13 +11,17 @@
 //     the reference by more than 2^8?") and never reduced, except for the first tile of an item
 //     and the rare tile that raises it; row sums stay in registers until the end.
 //
+// head_dim 64: a tile is one panel (16 KB for K, 16 KB for V) and O^T has M = 64, 16 rows in each quadrant's first lanes.
+// Half the bytes a tile, the same chain, so this one is bound by the chain and wants more CTAs (256 pairs of 64 rows
+// at 1000 keys: 20.9 us a layer, 3.5 TB/s; the mma.sync kernel took 29.3).
+//
 // Warps 0-7 (softmax): warp w reads lanes 32 (w % 4) .. + 31 (one key per thread) and half w / 4 of
 //   the rows; they also load Q.  P^T goes to shared memory as it lies in the registers: a key's
 //   probabilities are contiguous (the instruction's MN-major B operand).
-// Warp 8 (loader): K and V tiles (units K0 K1 V0 K2 V1 ...) into a ring of SLOTS 32 KB slots by TMA;
+// Warp 8 (loader): K and V tiles (units K0 K1 V0 K2 V1 ...) into a ring of SLOTS slots by TMA;
 //   the tile with the prefix end and the tree's rows by boxes of 32 and 8 rows, spread over the lanes (by
 //   16-byte cp.async this tile cost one warp 1.3 us to issue); rows of V that must not count are cleared.
-// Warp 9 (issuer): one thread issues S^T two tiles ahead and O^T += V^T P^T in order.
+// Warp 9 (issuer): one elected lane issues S^T two tiles ahead and O^T += V^T P^T in order.
 // Key splits of a cluster are merged through distributed shared memory: each CTA stages its O in fp32,
 // sends the rows to their owners by bulk copies, and the owner adds up.
 // Every wait is bounded: if one runs out the request is flagged TWIG_DEV_INTERNAL.
