@@ -743,12 +743,14 @@ extern "C" twig_status tree_verify_attention_ex(const void *q, const void *tree_
     //     128 rows x 250 10.6 / 11.3, 64 x 250 14.1 / 13.1
     //   head_dim 64 (up to 64 rows): 128 x 500 6.2 / 7.5 (12 rows), 9.2 / 8.3 (30 rows), 128 x 1000 10.5 / 9.2;
     //     64 x 1000 9.3 / 10.0, 64 x 2000 12.8 / 11.9; 256 x 250 7.5 / 6.9, 256 x 2000 58.8 / 43.4; 4 x 4000 7.6 / 7.2
+    // Up to 32 rows the line lies above the crossing: a cache is seldom full, and a short length in a large cache would
+    // pay for the wrong choice (32 pairs of 26 rows, 250 keys: 5.3 / 6.9).
     // (The persistent kernel measured slower on every shape tried, so it only runs when it is named.)
     const long long pairs = (long long)cache->batch * cache->n_kv_heads, keys = pairs * cache->max_len;
     bool big;
     if (cache->head_dim == 64) big = rows <= 64 && (keys >= (pairs > 148 ? 60000 : 100000) || cache->max_len >= 4000);
     else if (rows > 64) big = rows <= 128 || pairs * ((rows + 127) / 128) > 32 || cache->max_len > 256;
-    else big = pairs > 74 || cache->max_len >= 3000 || keys >= (rows > 32 ? 8000 : rows > 16 ? 16000 : 40000);
+    else big = pairs > 74 || cache->max_len >= 3000 || keys >= (rows > 32 ? 8000 : rows > 16 ? 32000 : 40000);
     if (big) {
       const twig_status us = launch_tree_attn_tcgen05(p, cache->batch, rows, st);
       if (us != TWIG_ERR_UNSUPPORTED) return us;     // no tensor map for this layout: the mma.sync kernel
